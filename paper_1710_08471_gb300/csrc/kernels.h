@@ -82,13 +82,22 @@ cudaError_t trmm_upper_small(int n, const double* A, int64_t lda, bool a_trans, 
                              double* C, int64_t ldc, cudaStream_t s);
 
 // ---------------------------------------------------------------- CholInv
-// [L, Y] = CholInv(W) (Algorithm 1): recursive halving with FP64 GEMMs and a
-// one-CTA base case of size <= 64. `work` and `U` are n x n scratch (ld n).
-constexpr int CHOLINV_BASE = 64;
+// [L, Y] = CholInv(W) (Algorithm 1): recursive halving with FP64 GEMMs and
+// one-launch leaves of size <= CHOLINV_LEAF. `work` and `U` are n x n scratch (ld n).
+constexpr int CHOLINV_BASE = 64;   // split points are multiples of this
+constexpr int CHOLINV_LEAF = 128;  // largest leaf
+// A leaf (n <= CHOLINV_LEAF), one cluster launch: writes the whole blocks of L
+// and Y (zeros above the diagonal) and, when given, R = L^T (zeros below) and
+// the Q-form's packed R^-1 in column groups of rpw (see pack_rinv_from_lower).
+// Only W's lower triangle is read, completely before anything is written, so W
+// may share storage with an output.
+cudaError_t cholinv_leaf(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
+                         double* Rt, int64_t ldrt, double* Rp, int rpw, DevStatus* st, int pass, long long off,
+                         cudaStream_t s);
 // ws (wsn doubles, may be null) is split-k scratch for the recursion's small
 // products; cholinv_splitk_doubles() is enough for any n.
 // With Rt, also R = L^T (ld ldrt, zeros below the diagonal); with Rp, also
-// the Q-form's packed R^-1 (pack_rinv_from_lower). At n = 64 one kernel writes
+// the Q-form's packed R^-1 (pack_rinv_from_lower). A leaf's kernel writes
 // everything; otherwise the transpose and the packing are launches of their own.
 cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                     double* work, double* U, DevStatus* st, int pass, cudaStream_t s, double* ws = nullptr,
