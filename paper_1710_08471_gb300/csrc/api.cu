@@ -32,7 +32,6 @@ struct cqr2_plan_st {
   cqr2_plan_st* pan_tail = nullptr;
   double* pan_C = nullptr;
   double* Tsolve = nullptr;  // block-substitution scratch, ldt x right_solve_temp_cols(n)
-  double* skws = nullptr;    // split-k scratch of CholInv's small products
   int64_t ldt = 0;
   int64_t oz_cap = 0;    // same for the split-precision Gram partials
   int precision = CQR2_FP64;
@@ -125,8 +124,7 @@ cudaError_t r_product(cqr2_plan_st* p, int n, const double* A, int64_t lda, bool
                       int64_t ldb, double* C, int64_t ldc, cudaStream_t s) {
   if (n <= TRMM_SMALL_MAX) return trmm_upper_small(n, A, lda, a_trans, B, ldb, C, ldc, s);
   return gemm_f64(n, n, n, 1.0, A, lda, B, ldb, 0.0, C, ldc,
-                  (a_trans ? GEMM_TA : 0u) | GEMM_A_UPPER | GEMM_B_UPPER | GEMM_C_UPPER | GEMM_BETA0, s, p->skws,
-                  cholinv_splitk_doubles());
+                  (a_trans ? GEMM_TA : 0u) | GEMM_A_UPPER | GEMM_B_UPPER | GEMM_C_UPPER | GEMM_BETA0, s);
 }
 
 // Copy a column-major rows x cols block: one linear copy when both sides are
@@ -197,13 +195,12 @@ cudaError_t plan_cholinv(cqr2_plan_st* p, int pass, cudaStream_t s, double* Rt =
   const int n = (int)p->n;
   if (p->inv_depth > 0) {
     cudaError_t e = cholinv_depth(n, p->W, n, p->L, n, p->Y, n, p->Wk, p->U, p->Tsolve, p->ldt, p->st, pass,
-                                  p->inv_depth, s, p->skws, cholinv_splitk_doubles());
+                                  p->inv_depth, s);
     if (e == cudaSuccess && Rt != nullptr) e = transpose_lower(p->L, n, n, Rt, n, s);
     if (e == cudaSuccess && Rp != nullptr) e = pack_rinv_from_lower(p->Y, n, n, Rp, s);
     return e;
   }
-  return cholinv(n, p->W, n, p->L, n, p->Y, n, p->Wk, p->U, p->st, pass, s, p->skws, cholinv_splitk_doubles(), Rt,
-                 n, Rp);
+  return cholinv(n, p->W, n, p->L, n, p->Y, n, p->Wk, p->U, p->st, pass, s, Rt, n, Rp);
 }
 
 // X = B R^-1 = B L^-T (general path, rows x n): one triangular multiply by
@@ -468,11 +465,9 @@ cqr2_status_t factor_panels(cqr2_plan_st* p, const double* dA, int64_t lda, doub
     if (dQ != dA) TRY(copy_cols(Qk, ldq, dA + c0 * lda, lda, m, bk, cudaMemcpyDeviceToDevice, s));
     if (c0 > 0) {
       double* Rk = dR + c0 * ldr;  // R(0:c0, c0:c0+bk)
-      TRY(gemm_f64(c0, bk, m, 1.0, dQ, ldq, Qk, ldq, 0.0, Rk, ldr, GEMM_TA | GEMM_BETA0, s, p->skws,
-                   cholinv_splitk_doubles()));
+      TRY(gemm_f64(c0, bk, m, 1.0, dQ, ldq, Qk, ldq, 0.0, Rk, ldr, GEMM_TA | GEMM_BETA0, s));
       TRY(gemm_f64(m, bk, c0, -1.0, dQ, ldq, Rk, ldr, 1.0, Qk, ldq, 0, s));
-      TRY(gemm_f64(c0, bk, m, 1.0, dQ, ldq, Qk, ldq, 0.0, p->pan_C, c0, GEMM_TA | GEMM_BETA0, s, p->skws,
-                   cholinv_splitk_doubles()));
+      TRY(gemm_f64(c0, bk, m, 1.0, dQ, ldq, Qk, ldq, 0.0, p->pan_C, c0, GEMM_TA | GEMM_BETA0, s));
       TRY(gemm_f64(m, bk, c0, -1.0, dQ, ldq, p->pan_C, c0, 1.0, Qk, ldq, 0, s));
       TRY(add_block(p->pan_C, c0, Rk, ldr, c0, bk, s));
     }
@@ -636,8 +631,6 @@ cqr2_status_t cqr2_plan_create(cqr2_plan_t* plan, int64_t m, int64_t n, int32_t 
     take((size_t)n * sizeof(int));                                   // 19 R^-1 exponents
     take((size_t)p->oz_cap * n * n * sizeof(double));                // 20 Gram partials
   }
-  const int i_sk = k;
-  take(cholinv_splitk_doubles() * sizeof(double));                   // split-k scratch of CholInv
   if (cudaMalloc(&p->ws, sz) != cudaSuccess) {
     cudaGetLastError();
     delete p;
@@ -665,7 +658,6 @@ cqr2_status_t cqr2_plan_create(cqr2_plan_t* plan, int64_t m, int64_t n, int32_t 
   p->Q1 = p->small ? nullptr : at(9);
   p->lspart = at(10);
   p->st = reinterpret_cast<DevStatus*>(p->ws + off[11]);
-  p->skws = at(i_sk);
   if (oz_S) {
     p->oz_planes = reinterpret_cast<unsigned short*>(p->ws + off[14]);
     p->oz_rinv = reinterpret_cast<unsigned short*>(p->ws + off[15]);
@@ -973,8 +965,7 @@ cqr2_status_t cqr2_cholinv(cqr2_plan_t p, const double* dW, int64_t ldw, double*
   cqr2_status_t r = check_device(p);
   if (r != CQR2_OK) return r;
   TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), p->stream));
-  TRY(cholinv((int)p->n, dW, ldw, dL, ldl, dY, ldy, p->Wk, p->U, p->st, 1, p->stream, p->skws,
-              cholinv_splitk_doubles()));
+  TRY(cholinv((int)p->n, dW, ldw, dL, ldl, dY, ldy, p->Wk, p->U, p->st, 1, p->stream));
   if (info) return read_info(p, info);
   return CQR2_OK;
 }

@@ -40,45 +40,44 @@ __global__ void k_copy_upper(const double* __restrict__ X, int64_t ldx, int n, d
 }
 
 cudaError_t rec(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, double* Y, int64_t ldy, double* U,
-                int64_t ldu, DevStatus* st, int pass, long long off, cudaStream_t s, double* ws, size_t wsn) {
+                int64_t ldu, DevStatus* st, int pass, long long off, cudaStream_t s) {
   if (n <= CHOLINV_LEAF) return cholinv_leaf(n, Wk, ldk, L, ldl, Y, ldy, nullptr, 0, nullptr, 0, st, pass, off, s);
   const int n1 = NB * (int)ceil_div(n, 2 * NB);
   const int n2 = n - n1;
   cudaError_t e;
   // [L11, Y11] = CholInv(W11)
-  if ((e = rec(n1, Wk, ldk, L, ldl, Y, ldy, U, ldu, st, pass, off, s, ws, wsn)) != cudaSuccess) return e;
+  if ((e = rec(n1, Wk, ldk, L, ldl, Y, ldy, U, ldu, st, pass, off, s)) != cudaSuccess) return e;
   // L21 = W21 Y11^T
   if ((e = gemm_f64(n2, n1, n1, 1.0, Wk + n1, ldk, Y, ldy, 0.0, L + n1, ldl, GEMM_TB | GEMM_B_UPPER | GEMM_BETA0,
-                    s, ws, wsn)) != cudaSuccess)
+                    s)) != cudaSuccess)
     return e;
   // W22 <- W22 - L21 L21^T (lower triangle)
   double* W22 = Wk + n1 + (int64_t)n1 * ldk;
-  if ((e = gemm_f64(n2, n2, n1, -1.0, L + n1, ldl, L + n1, ldl, 1.0, W22, ldk, GEMM_TB | GEMM_C_LOWER, s, ws,
-                    wsn)) != cudaSuccess)
+  if ((e = gemm_f64(n2, n2, n1, -1.0, L + n1, ldl, L + n1, ldl, 1.0, W22, ldk, GEMM_TB | GEMM_C_LOWER, s)) != cudaSuccess)
     return e;
   // [L22, Y22] = CholInv(W22 - L21 L21^T)
   double* L22 = L + n1 + (int64_t)n1 * ldl;
   double* Y22 = Y + n1 + (int64_t)n1 * ldy;
-  if ((e = rec(n2, W22, ldk, L22, ldl, Y22, ldy, U, ldu, st, pass, off + n1, s, ws, wsn)) != cudaSuccess) return e;
+  if ((e = rec(n2, W22, ldk, L22, ldl, Y22, ldy, U, ldu, st, pass, off + n1, s)) != cudaSuccess) return e;
   // U = L21 Y11
-  if ((e = gemm_f64(n2, n1, n1, 1.0, L + n1, ldl, Y, ldy, 0.0, U, ldu, GEMM_B_LOWER | GEMM_BETA0, s, ws, wsn)) !=
+  if ((e = gemm_f64(n2, n1, n1, 1.0, L + n1, ldl, Y, ldy, 0.0, U, ldu, GEMM_B_LOWER | GEMM_BETA0, s)) !=
       cudaSuccess)
     return e;
   // Y21 = -Y22 U
-  return gemm_f64(n2, n1, n2, -1.0, Y22, ldy, U, ldu, 0.0, Y + n1, ldy, GEMM_A_LOWER | GEMM_BETA0, s, ws, wsn);
+  return gemm_f64(n2, n1, n2, -1.0, Y22, ldy, U, ldu, 0.0, Y + n1, ldy, GEMM_A_LOWER | GEMM_BETA0, s);
 }
 
 // Depth-limited recursion: the top `depth` levels form L21 by block forward
 // substitution through the diagonal blocks' inverses and leave Y21 zero.
 cudaError_t rec_depth(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, double* Y, int64_t ldy, double* U,
                       int64_t ldu, double* T, int64_t ldt, DevStatus* st, int pass, long long off, int depth,
-                      cudaStream_t s, double* ws, size_t wsn) {
-  if (depth <= 0 || n <= NB) return rec(n, Wk, ldk, L, ldl, Y, ldy, U, ldu, st, pass, off, s, ws, wsn);
+                      cudaStream_t s) {
+  if (depth <= 0 || n <= NB) return rec(n, Wk, ldk, L, ldl, Y, ldy, U, ldu, st, pass, off, s);
   const int n1 = NB * (int)ceil_div(n, 2 * NB);
   const int n2 = n - n1;
   cudaError_t e;
   // [L11, Y11] with Y11 known on its leaf blocks only
-  if ((e = rec_depth(n1, Wk, ldk, L, ldl, Y, ldy, U, ldu, T, ldt, st, pass, off, depth - 1, s, ws, wsn)) !=
+  if ((e = rec_depth(n1, Wk, ldk, L, ldl, Y, ldy, U, ldu, T, ldt, st, pass, off, depth - 1, s)) !=
       cudaSuccess)
     return e;
   // L21 = W21 L11^-T
@@ -86,11 +85,10 @@ cudaError_t rec_depth(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, do
     return e;
   // W22 <- W22 - L21 L21^T (lower triangle)
   double* W22 = Wk + n1 + (int64_t)n1 * ldk;
-  if ((e = gemm_f64(n2, n2, n1, -1.0, L + n1, ldl, L + n1, ldl, 1.0, W22, ldk, GEMM_TB | GEMM_C_LOWER, s, ws,
-                    wsn)) != cudaSuccess)
+  if ((e = gemm_f64(n2, n2, n1, -1.0, L + n1, ldl, L + n1, ldl, 1.0, W22, ldk, GEMM_TB | GEMM_C_LOWER, s)) != cudaSuccess)
     return e;
   return rec_depth(n2, W22, ldk, L + n1 + (int64_t)n1 * ldl, ldl, Y + n1 + (int64_t)n1 * ldy, ldy, U, ldu, T, ldt,
-                   st, pass, off + n1, depth - 1, s, ws, wsn);
+                   st, pass, off + n1, depth - 1, s);
 }
 
 }  // namespace
@@ -126,17 +124,12 @@ cudaError_t right_solve(int64_t M, int N, const double* B, int64_t ldb, double* 
                      depth - 1, T, ldt, s);
 }
 
-// Split-k partials of one product: ks * M * N with ks * tiles <= SMs, so 256
-// SMs' worth of 64 x 64 tiles is enough for any size (the GEMM lowers ks
-// further if the scratch is short).
-size_t cholinv_splitk_doubles() { return (size_t)256 * 64 * 64; }
-
 int right_solve_temp_cols(int n) { return n <= NB ? n : NB * (int)ceil_div(n, 2 * NB); }
 
 cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                           double* work, double* U, double* T, int64_t ldt, DevStatus* st, int pass, int depth,
-                          cudaStream_t s, double* ws, size_t wsn) {
-  if (depth <= 0) return cholinv(n, W, ldw, L, ldl, Y, ldy, work, U, st, pass, s, ws, wsn);
+                          cudaStream_t s) {
+  if (depth <= 0) return cholinv(n, W, ldw, L, ldl, Y, ldy, work, U, st, pass, s);
   cudaError_t e;
   if ((e = cudaMemcpy2DAsync(work, (size_t)n * sizeof(double), W, (size_t)ldw * sizeof(double),
                              (size_t)n * sizeof(double), (size_t)n, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
@@ -147,11 +140,11 @@ cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_
   if ((e = cudaMemset2DAsync(Y, (size_t)ldy * sizeof(double), 0, (size_t)n * sizeof(double), (size_t)n, s)) !=
       cudaSuccess)
     return e;
-  return rec_depth(n, work, n, L, ldl, Y, ldy, U, n, T, ldt, st, pass, 0, depth, s, ws, wsn);
+  return rec_depth(n, work, n, L, ldl, Y, ldy, U, n, T, ldt, st, pass, 0, depth, s);
 }
 
 cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
-                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s, double* ws, size_t wsn,
+                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s,
                     double* Rt, int64_t ldrt, double* Rp) {
   cudaError_t e;
   if (n <= CHOLINV_LEAF) {
@@ -174,7 +167,7 @@ cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl,
   if ((e = cudaMemset2DAsync(Y, (size_t)ldy * sizeof(double), 0, (size_t)n * sizeof(double), (size_t)n, s)) !=
       cudaSuccess)
     return e;
-  if ((e = rec(n, work, n, L, ldl, Y, ldy, U, n, st, pass, 0, s, ws, wsn)) != cudaSuccess) return e;
+  if ((e = rec(n, work, n, L, ldl, Y, ldy, U, n, st, pass, 0, s)) != cudaSuccess) return e;
   if (Rt != nullptr && (e = transpose_lower(L, ldl, n, Rt, ldrt, s)) != cudaSuccess) return e;
   if (Rp != nullptr) return pack_rinv_from_lower(Y, ldy, n, Rp, s);
   return cudaSuccess;

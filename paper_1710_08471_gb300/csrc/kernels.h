@@ -68,12 +68,11 @@ enum : unsigned {
   GEMM_C_UPPER = 1u << 7,   // only C(i,j), i <= j, is computed; i > j written as 0
   GEMM_BETA0 = 1u << 8,     // C is not read (beta = 0)
 };
-// With scratch ws (ws_doubles doubles), a product too small to fill the GPU
-// splits k over up to 8 CTAs per tile and sums the partials in a fixed order
-// (deterministic; ws must not alias A, B or C).
+// A product too small to fill the GPU splits k over a cluster of up to 8 CTAs
+// per tile, whose partial sums are added in a fixed order (deterministic).
 cudaError_t gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda,
                      const double* B, int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags,
-                     cudaStream_t s, double* ws = nullptr, size_t ws_doubles = 0);
+                     cudaStream_t s);
 
 // R = op(A) B for upper-triangular n x n factors, n <= TRMM_SMALL_MAX, one
 // launch; op(A) = A^T (A lower) when a_trans. C below the diagonal is zeroed.
@@ -94,22 +93,18 @@ constexpr int CHOLINV_LEAF = 128;  // largest leaf
 cudaError_t cholinv_leaf(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                          double* Rt, int64_t ldrt, double* Rp, int rpw, DevStatus* st, int pass, long long off,
                          cudaStream_t s);
-// ws (wsn doubles, may be null) is split-k scratch for the recursion's small
-// products; cholinv_splitk_doubles() is enough for any n.
 // With Rt, also R = L^T (ld ldrt, zeros below the diagonal); with Rp, also
 // the Q-form's packed R^-1 (pack_rinv_from_lower). A leaf's kernel writes
 // everything; otherwise the transpose and the packing are launches of their own.
 cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
-                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s, double* ws = nullptr,
-                    size_t wsn = 0, double* Rt = nullptr, int64_t ldrt = 0, double* Rp = nullptr);
-size_t cholinv_splitk_doubles();
+                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s, double* Rt = nullptr, int64_t ldrt = 0, double* Rp = nullptr);
 // Inverse depth (the paper's triangular inverted blocks): the top `depth`
 // halvings form L21 = W21 L11^-T by block forward substitution and leave Y21
 // zero, so Y holds the inverses of L's diagonal blocks only. T is scratch of
 // n x right_solve_temp_cols(n) doubles (ld ldt >= n).
 cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                           double* work, double* U, double* T, int64_t ldt, DevStatus* st, int pass, int depth,
-                          cudaStream_t s, double* ws = nullptr, size_t wsn = 0);
+                          cudaStream_t s);
 // X = B L^-T (M x N) for lower-triangular L whose diagonal-block inverses of a
 // depth-`depth` halving are in Y: X1 = B1 L11^-T, X2 = (B2 - X1 L21^T) L22^-T.
 // X may equal B. T is scratch of M x right_solve_temp_cols(N) (ld ldt >= M).
