@@ -163,7 +163,8 @@ cqr2_status_t cqr2_lstsq_rows(cqr2_plan_t plan, int64_t m, const double* dA, int
                               double* dx, double* dQ, int64_t ldq, double* dR, int64_t ldr, cqr2_info_t* info);
 
 /* Tuning knobs of a plan (set by the autotuner, cqr2_autotune, or by hand):
- * the number of Gram CTAs per SM (1..8, default 4), and whether to fuse the
+ * the largest number of Gram CTAs per SM (1..8, default 4; the library uses
+ * fewer where more would not help), and whether to fuse the
  * pass-1 Q-form with the pass-2 Gram (honoured only where CQR2_FUSED is). */
 cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t plan, int32_t ctas_per_sm);
 cqr2_status_t cqr2_plan_set_fused(cqr2_plan_t plan, int32_t fused);

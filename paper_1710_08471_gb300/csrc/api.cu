@@ -39,6 +39,7 @@ struct cqr2_plan_st {
   int device = 0;
   cudaStream_t stream = nullptr;
   GramGeom g;
+  GramGeom gf;  // the fused Q-form + Gram's row ranges (whole 32-row panels)
   bool small = false;  // n <= 256: panel Q-form kernel, Q1 staged in the output Q
   bool fused = false;  // CQR2_FUSED requested and n small enough to fuse
   int64_t gemv_nsplit = 0;
@@ -237,6 +238,7 @@ cqr2_status_t set_rows(cqr2_plan_st* p, int64_t m) {
   if (m < p->n || m > p->m) return CQR2_ERR_INVALID_ARG;
   if (m == p->cm) return CQR2_OK;
   p->g = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps);
+  p->gf = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps, QFORM_PANEL);
   p->gemv_nsplit = gemv_splits(m, (int)p->n);
   if (p->oz_S && ozaki_make_maps(p->oz_maps, m, (int)p->n, p->oz_Scap, p->oz_planes, p->oz_rinv) != cudaSuccess) {
     p->cm = 0;
@@ -381,7 +383,7 @@ cqr2_status_t factor_impl(cqr2_plan_st* p, const double* dA, int64_t lda, double
     Stage st(p, CQR2_STAGE_QFORM1);
     if (p->fused) {
       // Q1 and the partial Grams of Q1 in one sweep over A
-      TRY(qform_gram_small(dA, lda, p->cm, n, p->Rp, dQ, ldq, p->g, p->partial, s));
+      TRY(qform_gram_small(dA, lda, p->cm, n, p->Rp, dQ, ldq, p->gf, p->partial, s));
     } else {
       TRY(qform_small(dA, lda, p->cm, n, p->Rp, dQ, ldq, s));
     }
@@ -394,7 +396,7 @@ cqr2_status_t factor_impl(cqr2_plan_st* p, const double* dA, int64_t lda, double
   {
     Stage st(p, CQR2_STAGE_GRAM2);
     if (!p->fused) TRY(gram_partials(X2, ldx2, p->cm, n, p->g, p->partial, s));
-    TRY(gram_reduce(p->partial, p->g, n, p->W, n, s));
+    TRY(gram_reduce(p->partial, p->fused ? p->gf : p->g, n, p->W, n, s));
   }
   {
     Stage st(p, CQR2_STAGE_CHOLINV2);
@@ -679,6 +681,7 @@ cqr2_status_t cqr2_plan_create(cqr2_plan_t* plan, int64_t m, int64_t n, int32_t 
     }
   }
   p->g = gram_geometry(m, (int)n, p->gram_cap, p->gram_cps);
+  p->gf = gram_geometry(m, (int)n, p->gram_cap, p->gram_cps, QFORM_PANEL);
   p->cm = m;  // geometry and tensor maps above are for the full row count
   std::memset(p->h_st, 0, sizeof(DevStatus));
   if (cudaMemsetAsync(p->st, 0, sizeof(DevStatus), p->stream) != cudaSuccess) {

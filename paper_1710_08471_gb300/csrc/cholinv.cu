@@ -153,8 +153,8 @@ cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl,
     // is a launch of its own over the whole GPU
     double* leafRp = n <= NB ? Rp : nullptr;
     const int rpw = leafRp != nullptr ? qform_group_width(n) : 0;
-    // the packing's layout is the Q-form's: the same number of column groups
-    if (leafRp != nullptr && rpack_doubles(n) != (size_t)RP_GROUPS * n * rpw) return cudaErrorInvalidValue;
+    // the packing's layout is the Q-form's: the same number of column groups and pitch
+    if (leafRp != nullptr && rpack_doubles(n) != (size_t)RP_GROUPS * n * (rpw + (rpw & 1))) return cudaErrorInvalidValue;
     if ((e = cholinv_leaf(n, W, ldw, L, ldl, Y, ldy, Rt, ldrt, leafRp, rpw, st, pass, 0, s)) != cudaSuccess) return e;
     return Rp != nullptr && leafRp == nullptr ? pack_rinv_from_lower(Y, ldy, n, Rp, s) : cudaSuccess;
   }

@@ -236,7 +236,8 @@ __global__ void __launch_bounds__(LT, 1)
   __shared__ int s_exact;  // a pivot of the panel factored last needs real divisions
   const int C = (int)cluster_size(), me = (int)cluster_rank();
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31, r = lane & 7, g = lane >> 3;
-  const int nb = (n + TB - 1) / TB;
+  const int nb = (n + TB - 1) / TB, rpp = rpw + (rpw & 1);
+  const int rpl = rpw > 0 ? (n + rpw - 1) / rpw * rpw - n : 0;  // R^-1's packing: pitch rpp, the first group lacks rpl columns
   // own block columns: q-th is q C + (q even ? me : C - 1 - me)
   auto column = [&](int q) { return q * C + ((q & 1) ? C - 1 - me : me); };
   auto owner = [&](int j) {
@@ -397,9 +398,9 @@ __global__ void __launch_bounds__(LT, 1)
         if (i > j && Rt != nullptr) Rt[i + (int64_t)j * ldrt] = 0.0;
       }
       if (Rp != nullptr)
-        for (int e = who; e < RP_GROUPS * n * rpw; e += stride) {
-          const int c = e % rpw, k = (e / rpw) % n, col = (e / (rpw * n)) * rpw + c;
-          if (col >= n || k > col) Rp[e] = 0.0;
+        for (int e = who; e < RP_GROUPS * n * rpp; e += stride) {
+          const int c = e % rpp, k = (e / rpp) % n, col = (e / (rpp * n)) * rpw + c - rpl;
+          if (c >= rpw || col < 0 || col >= n || k > col) Rp[e] = 0.0;
         }
     }
   }
@@ -450,7 +451,7 @@ __global__ void __launch_bounds__(LT, 1)
           if (gj > gi) continue;
           const double y = (h ? v.y : v.x) * s;
           Y[gi + (int64_t)gj * ldy] = y;
-          if (Rp != nullptr) Rp[((int64_t)(gi / rpw) * n + gj) * rpw + gi % rpw] = y;  // R^-1(gj, gi)
+          if (Rp != nullptr) Rp[((int64_t)((gi + rpl) / rpw) * n + gj) * rpp + (gi + rpl) % rpw] = y;  // R^-1(gj, gi)
         }
       }
     }

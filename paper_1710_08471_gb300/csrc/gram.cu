@@ -1,23 +1,28 @@
 // Split-m Gram (Syrk, Section II-A; Algorithm CQR step 1): W = A^T A.
 //
 // The n x n upper triangle is cut into T x T tiles (diagonal and strictly
-// upper). Each CTA owns one tile and one contiguous range of rows of A and
-// accumulates that range's partial tile in registers; a second kernel sums the
-// ranges' partials in a fixed order (deterministic), which is the one-GPU
-// counterpart of the 1D algorithm's local Syrk + Allreduce (Algorithm 1D-CQR).
+// upper), T at most 128 and chosen so that the tiles are nearly equal (the
+// last ones narrower). A CTA owns one range of rows of A and one off-diagonal
+// tile or two diagonal ones (about the same work) and accumulates the range's
+// partial tiles in registers; a second kernel sums the ranges' partials in a
+// fixed order (deterministic), which is the one-GPU counterpart of the 1D
+// algorithm's local Syrk + Allreduce (Algorithm 1D-CQR).
 //
 // GB300 FP64 runs at about 2 FMA per clock per SM and a warp instruction pays
-// for all 32 lanes whether or not they are active, so the diagonal tiles use a
-// flattened list of the T(T+1)/2 upper pairs (no lane computes a pair below
-// the diagonal) and off-diagonal tiles give each lane one column j and a
-// strided set of rows i (the row operand is a shared-memory broadcast).
+// for all 32 lanes whether or not they are active, so no slot is spent on
+// padding: diagonal tiles use the flattened list of their upper pairs
+// (gram_pairs.cuh), off-diagonal tiles give each lane one column of the first
+// block (T is a multiple of 16, so two lanes per column fill whole warps) and
+// every second row of the other (a shared-memory broadcast), and the row
+// ranges are cut so that the CTAs, all of equal work, fill whole waves.
 // Row panels of KC rows are staged through double-buffered shared memory with
-// cp.async; the layout [row][column] (padded) makes lanes that differ in the
-// column index hit distinct banks.
+// cp.async; the layout [row][column] (odd pitch) makes the copies' lanes, which
+// differ in the row, hit distinct banks.
 #include <algorithm>
 #include <mutex>
 
 #include "../../include/cqr2.h"
+#include "gram_pairs.cuh"
 #include "kernels.h"
 
 namespace cqr2 {
@@ -34,128 +39,138 @@ constexpr int KC = 32;  // rows per staged chunk
 constexpr size_t NOALLOC_DOUBLES = CQR2_NOALLOC_SCRATCH_BYTES / sizeof(double);
 static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_DOUBLES];
 
-template <int T>
-__host__ __device__ constexpr int lds() {
-  return T + 1;
+constexpr int NT = GRAM_NT;
+
+// Rows [r0, r1) of columns c0 .. c0 + w - 1 into X[row][column], zeros past r1.
+__device__ __forceinline__ void load_chunk(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int c0,
+                                           int w, double* X, int pitch) {
+  const int kk = threadIdx.x % KC;
+  const int64_t row = r0 + kk;
+  const bool ok = row < r1;
+  const double* src = A + (ok ? row : 0) + (int64_t)c0 * lda;
+#pragma unroll 4
+  for (int c = threadIdx.x / KC; c < w; c += NT / KC) cp_async8(X + kk * pitch + c, src + (int64_t)c * lda, ok ? 8 : 0);
 }
 
-template <int T, int NT, bool DIAG>
-__global__ void __launch_bounds__(NT) k_gram_tile(const double* __restrict__ A, int64_t lda, int64_t m, int n,
-                                                  int64_t rows_per_split, int ntile, int ntiles_total,
-                                                  double* __restrict__ partial) {
-  constexpr int LDS = lds<T>();
-  constexpr int NBLK = DIAG ? 1 : 2;
-  constexpr int P = DIAG ? T * (T + 1) / 2 : T * T;
-  constexpr int S = (P + NT - 1) / NT;
-  constexpr int STEP = NT / T;  // off-diagonal: row stride between a lane's slots
-  constexpr int E = KC * T / NT;  // elements per thread per block per chunk
-  static_assert((KC * T) % NT == 0, "chunk must split evenly");
-  static_assert(DIAG || (NT % T == 0), "off-diagonal mapping needs NT multiple of T");
-  extern __shared__ double smem[];
+// One diagonal tile of width w at column c0 over rows [r0, r1).
+template <int MAXS>
+__device__ __forceinline__ void diag_item(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int c0, int w,
+                                          double* smem, double* __restrict__ out, int T) {
+  const int pitch = w | 1;
+  GramPairs<MAXS> pairs;
+  pairs.init(threadIdx.x, w);
+  double* cur = smem;
+  double* nxt = smem + KC * pitch;
+  load_chunk(A, lda, r0, r1, c0, w, cur, pitch);
+  cp_async_commit();
+  for (int64_t r = r0; r < r1; r += KC) {
+    if (r + KC < r1) load_chunk(A, lda, r + KC, r1, c0, w, nxt, pitch);
+    cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+    pairs.add(cur, pitch, (int)min((int64_t)KC, (r1 - r + 3) & ~(int64_t)3));
+    __syncthreads();
+    double* x = cur;
+    cur = nxt;
+    nxt = x;
+  }
+  pairs.store(out, T);
+}
 
-  const int t = threadIdx.x;
-  int I, J, tile_index;
-  if (DIAG) {
-    I = J = blockIdx.y;
-    tile_index = I;
-  } else {
-    int rem = blockIdx.y;
-    I = 0;
+// The off-diagonal tile of columns cI .. cI + T - 1 and cJ .. cJ + wJ - 1
+// (wJ <= T) over rows [r0, r1): lane column i = t % T of the first block,
+// columns t / T, t / T + 2, ... of the second.
+template <int S>
+__device__ __forceinline__ void off_item(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int cI, int cJ,
+                                         int wJ, double* smem, double* __restrict__ out, int T) {
+  const int t = threadIdx.x, pitch = T | 1, i = t % T, jh = t / T;
+  const bool live = jh < 2;  // whole warps: T is a multiple of 16
+  double acc[S];
+#pragma unroll
+  for (int s = 0; s < S; ++s) acc[s] = 0.0;
+  double* cur = smem;
+  double* nxt = smem + 2 * KC * pitch;
+  load_chunk(A, lda, r0, r1, cI, T, cur, pitch);
+  load_chunk(A, lda, r0, r1, cJ, wJ, cur + KC * pitch, pitch);
+  cp_async_commit();
+  for (int64_t r = r0; r < r1; r += KC) {
+    if (r + KC < r1) {
+      load_chunk(A, lda, r + KC, r1, cI, T, nxt, pitch);
+      load_chunk(A, lda, r + KC, r1, cJ, wJ, nxt + KC * pitch, pitch);
+    }
+    cp_async_commit();
+    cp_async_wait<1>();
+    __syncthreads();
+    if (live) {
+      const int rows = (int)min((int64_t)KC, (r1 - r + 3) & ~(int64_t)3);
+      const double* X = cur + i;
+      const double* Y = cur + KC * pitch + jh;
+      for (int k = 0; k < rows; k += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const double x = X[(k + u) * pitch];
+          const double* y = Y + (k + u) * pitch;
+          // columns past wJ read stale staging words; they are not stored
+#pragma unroll
+          for (int s = 0; s < S; ++s) acc[s] = fma(x, y[2 * s], acc[s]);
+        }
+    }
+    __syncthreads();
+    double* x = cur;
+    cur = nxt;
+    nxt = x;
+  }
+  if (live)
+#pragma unroll
+    for (int s = 0; s < S; ++s)
+      if (jh + 2 * s < wJ) out[i + (jh + 2 * s) * T] = acc[s];
+}
+
+// One diagonal tile (n <= 128) of at most MAXS slots per thread.
+template <int MAXS>
+__global__ void __launch_bounds__(NT, MAXS <= 8 ? 3 : (MAXS <= 16 ? 2 : 1))
+    k_gram_diag(const double* __restrict__ A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T,
+                double* __restrict__ partial) {
+  extern __shared__ double smem[];
+  const int64_t r0 = (int64_t)blockIdx.x * rows_per_split, r1 = min(m, r0 + rows_per_split);
+  diag_item<MAXS>(A, lda, r0, r1, 0, n, smem, partial + (int64_t)blockIdx.x * T * T, T);
+}
+
+// Several tiles: blockIdx.y < noff takes an off-diagonal tile, the others two
+// diagonal ones in turn.
+__global__ void __launch_bounds__(NT, 1)
+    k_gram_tiles(const double* __restrict__ A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T, int ntile,
+                 int ntiles_total, double* __restrict__ partial) {
+  extern __shared__ double smem[];
+  const int64_t r0 = (int64_t)blockIdx.x * rows_per_split, r1 = min(m, r0 + rows_per_split);
+  double* out = partial + (int64_t)blockIdx.x * ntiles_total * (int64_t)(T * T);
+  const int noff = ntiles_total - ntile;
+  if ((int)blockIdx.y < noff) {
+    int rem = blockIdx.y, I = 0;
     while (rem >= ntile - 1 - I) {
       rem -= ntile - 1 - I;
       ++I;
     }
-    J = I + 1 + rem;
-    tile_index = ntile + blockIdx.y;
-  }
-  const int cI = I * T, cJ = J * T;
-  const int64_t r_begin = (int64_t)blockIdx.x * rows_per_split;
-  const int64_t r_end = min(m, r_begin + rows_per_split);
-
-  // Slot -> (i, j) inside the tile.
-  int oi[DIAG ? S : 1], oj[DIAG ? S : 1];
-  bool last_ok = true;
-  if (DIAG) {
-    int i = 0, start = 0;  // start = first flattened index of row i
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      int p = t + s * NT;
-      if (p >= P) {
-        p = P - 1;
-        last_ok = false;
-      }
-      while (p >= start + (T - i)) {
-        start += T - i;
-        ++i;
-      }
-      oi[s] = i;
-      oj[s] = i + (p - start);
+    const int J = I + 1 + rem, wJ = min(T, n - J * T);
+    double* o = out + (int64_t)(ntile + blockIdx.y) * (T * T);
+    // accumulators for 16, 32, ... columns of the narrower last block
+    switch ((wJ + 15) / 16) {
+      case 1: off_item<8>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 2: off_item<16>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 3: off_item<24>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 4: off_item<32>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 5: off_item<40>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 6: off_item<48>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      case 7: off_item<56>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
+      default: off_item<64>(A, lda, r0, r1, I * T, J * T, wJ, smem, o, T); break;
     }
+    return;
   }
-  const int jcol = t % T;       // off-diagonal lane column
-  const int irow0 = t / T;      // off-diagonal first row
-
-  double acc[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) acc[s] = 0.0;
-
-  auto load_chunk = [&](int buf, int64_t r0) {
-#pragma unroll
-    for (int blk = 0; blk < NBLK; ++blk) {
-      const int cbase = blk ? cJ : cI;
-      double* dst = smem + (size_t)((buf * NBLK + blk) * KC) * LDS;
-#pragma unroll
-      for (int q = 0; q < E; ++q) {
-        const int e = t + q * NT;
-        const int kk = e % KC, c = e / KC;
-        const int64_t row = r0 + kk;
-        const int col = cbase + c;
-        const bool ok = (row < r_end) && (col < n);
-        const double* src = ok ? (A + row + (int64_t)col * lda) : A;
-        cp_async8(dst + kk * LDS + c, src, ok ? 8 : 0);
-      }
-    }
-  };
-
-  const int64_t nchunks = r_end > r_begin ? (r_end - r_begin + KC - 1) / KC : 0;
-  if (nchunks > 0) load_chunk(0, r_begin);
-  cp_async_commit();
-  for (int64_t ch = 0; ch < nchunks; ++ch) {
-    const int buf = (int)(ch & 1);
-    if (ch + 1 < nchunks) load_chunk(buf ^ 1, r_begin + (ch + 1) * KC);
-    cp_async_commit();
-    cp_async_wait<1>();
+  const int d0 = 2 * ((int)blockIdx.y - noff);
+  for (int d = d0; d < min(d0 + 2, ntile); ++d) {
+    const int w = min(T, n - d * T);
     __syncthreads();
-    const double* As = smem + (size_t)(buf * NBLK * KC) * LDS;
-    if (DIAG) {
-#pragma unroll 4
-      for (int kk = 0; kk < KC; ++kk) {
-        const double* row = As + kk * LDS;
-#pragma unroll
-        for (int s = 0; s < S; ++s) acc[s] = fma(row[oi[s]], row[oj[s]], acc[s]);
-      }
-    } else {
-      const double* Bs = As + KC * LDS;
-#pragma unroll 4
-      for (int kk = 0; kk < KC; ++kk) {
-        const double bj = Bs[kk * LDS + jcol];
-        const double* arow = As + kk * LDS + irow0;
-#pragma unroll
-        for (int s = 0; s < S; ++s) acc[s] = fma(arow[s * STEP], bj, acc[s]);
-      }
-    }
-    __syncthreads();
-  }
-
-  double* out = partial + ((int64_t)blockIdx.x * ntiles_total + tile_index) * (int64_t)(T * T);
-  if (DIAG) {
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      if (s < S - 1 || last_ok) out[oi[s] + oj[s] * T] = acc[s];
-    }
-  } else {
-#pragma unroll
-    for (int s = 0; s < S; ++s) out[(irow0 + s * STEP) + jcol * T] = acc[s];
+    diag_item<gram_slots(128)>(A, lda, r0, r1, d * T, w, smem, out + (int64_t)d * (T * T), T);
   }
 }
 
@@ -183,7 +198,15 @@ __global__ void __launch_bounds__(32 * GRAM_RC) k_gram_reduce(const double* __re
     const int64_t stride = (int64_t)ntiles_total * T * T;
     const double* p = partial + (int64_t)tile * T * T + loc;
     const int64_t b0 = nsplit * c / GRAM_RC, b1 = nsplit * (c + 1) / GRAM_RC;
-    for (int64_t b = b0; b < b1; ++b) s += p[b * stride];
+    int64_t b = b0;
+    for (; b + 8 <= b1; b += 8) {  // eight loads in flight
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = p[(b + u) * stride];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; b < b1; ++b) s += p[b * stride];
   }
   part[c][lane] = s;
   __syncthreads();
@@ -196,62 +219,67 @@ __global__ void __launch_bounds__(32 * GRAM_RC) k_gram_reduce(const double* __re
   }
 }
 
-template <int T, int NT, bool DIAG>
-size_t gram_smem() {
-  return (size_t)2 * (DIAG ? 1 : 2) * KC * lds<T>() * sizeof(double);
-}
-
-template <int T, int NT, bool DIAG>
-cudaError_t launch_tile(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,
-                        int ntiles_y, cudaStream_t s) {
-  if (ntiles_y == 0) return cudaSuccess;
-  const size_t sm = gram_smem<T, NT, DIAG>();
-  auto kern = k_gram_tile<T, NT, DIAG>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+template <int MAXS>
+cudaError_t launch_diag(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,
+                        cudaStream_t s) {
+  const size_t sm = (size_t)2 * KC * (n | 1) * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(k_gram_diag<MAXS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(2 * KC * 129 * sizeof(double)));
   if (e != cudaSuccess) return e;
-  dim3 grid((unsigned)g.nsplit, (unsigned)ntiles_y);
-  kern<<<grid, NT, sm, s>>>(A, lda, m, n, g.rows_per_split, g.ntile, g.ntiles_total, partial);
+  k_gram_diag<MAXS><<<(unsigned)g.nsplit, NT, sm, s>>>(A, lda, m, n, g.rows_per_split, g.T, partial);
   count_launch();
   return cudaGetLastError();
 }
 
 }  // namespace
 
-GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm) {
+GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, int row_unit) {
   GramGeom g;
-  g.T = n <= 32 ? 32 : (n <= 64 ? 64 : 128);
-  g.ntile = (int)ceil_div(n, g.T);
+  g.ntile = (int)ceil_div(n, 128);
+  g.T = (int)ceil_div(ceil_div(n, g.ntile), 16) * 16;
   g.ntiles_total = g.ntile + g.ntile * (g.ntile - 1) / 2;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // About ctas_per_sm CTAs per SM in total, but never a range shorter than one chunk.
-  int64_t want = std::max<int64_t>(1, ceil_div((int64_t)std::max(1, ctas_per_sm) * sms, g.ntiles_total));
-  want = std::min<int64_t>(want, std::max<int64_t>(1, ceil_div(m, KC)));
+  // CTAs of equal work per row range: one per off-diagonal tile, one per two
+  // diagonal tiles.
+  const int64_t items = g.ntiles_total - g.ntile + ceil_div(g.ntile, 2);
+  // CTAs per SM: one, and where several are resident at a time (few slots per
+  // thread) and each still has 35000 clocks (17 us) of FP64 work, that many.
+  // More only cost: filling a CTA's pipeline, writing its partial tiles and
+  // reading them back take 2 to 3 us. Gram and sum together with 1, 2, 3, 4
+  // CTAs per SM: 4096 x 64 29, 32, 41, 41 us; 50021 x 100 435, 451, 463, 474 us;
+  // 131072 x 32 166, 145, 136, 171 us; 262144 x 16 105, 93, 89, 125 us.
+  const int slots = gram_slots((int)std::min<int64_t>(n, 128));
+  const int resident = slots <= 8 ? 3 : (slots <= 16 ? 2 : 1);
+  const double clocks = (double)m * n * (n + 1) / 2 / (2.0 * sms);
+  const int64_t per_sm = std::min<int64_t>(std::max(1, ctas_per_sm), clocks >= 35000.0 * resident ? resident : 1);
+  // as many ranges as fit in that many whole waves, none shorter than 8 rows
+  int64_t want = std::max<int64_t>(1, per_sm * sms / items);
+  want = std::min<int64_t>(want, std::max<int64_t>(1, m / 8));
   if (max_splits > 0) want = std::min<int64_t>(want, max_splits);
-  g.rows_per_split = ceil_div(ceil_div(m, want), KC) * KC;
+  g.rows_per_split = ceil_div(ceil_div(m, want), row_unit) * row_unit;
   g.nsplit = std::max<int64_t>(1, ceil_div(m, g.rows_per_split));
   return g;
 }
 
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,
                           cudaStream_t s) {
-  const int noff = g.ntiles_total - g.ntile;
-  cudaError_t e;
-  switch (g.T) {
-    case 32:
-      e = launch_tile<32, 128, true>(A, lda, m, n, g, partial, g.ntile, s);
-      if (e == cudaSuccess) e = launch_tile<32, 128, false>(A, lda, m, n, g, partial, noff, s);
-      return e;
-    case 64:
-      e = launch_tile<64, 256, true>(A, lda, m, n, g, partial, g.ntile, s);
-      if (e == cudaSuccess) e = launch_tile<64, 256, false>(A, lda, m, n, g, partial, noff, s);
-      return e;
-    default:
-      e = launch_tile<128, 256, true>(A, lda, m, n, g, partial, g.ntile, s);
-      if (e == cudaSuccess) e = launch_tile<128, 256, false>(A, lda, m, n, g, partial, noff, s);
-      return e;
+  if (g.ntile == 1) {
+    const int slots = gram_slots(n);
+    if (slots <= 8) return launch_diag<8>(A, lda, m, n, g, partial, s);
+    if (slots <= 16) return launch_diag<16>(A, lda, m, n, g, partial, s);
+    if (slots <= 24) return launch_diag<24>(A, lda, m, n, g, partial, s);
+    return launch_diag<gram_slots(128)>(A, lda, m, n, g, partial, s);
   }
+  constexpr size_t sm = (size_t)4 * KC * 129 * sizeof(double);
+  cudaError_t e = cudaFuncSetAttribute(k_gram_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  const int noff = g.ntiles_total - g.ntile;
+  dim3 grid((unsigned)g.nsplit, (unsigned)(noff + ceil_div(g.ntile, 2)));
+  k_gram_tiles<<<grid, NT, sm, s>>>(A, lda, m, n, g.rows_per_split, g.T, g.ntile, g.ntiles_total, partial);
+  count_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw, cudaStream_t s) {

@@ -21,15 +21,16 @@ int64_t launch_count();
 // ranges whose partial Grams are summed in a fixed order, the single-GPU form
 // of the 1D algorithm's Allreduce, Algorithm 1D-CQR).
 struct GramGeom {
-  int T = 0;              // output tile width (32, 64 or 128)
+  int T = 0;              // output tile width, a multiple of 16 up to 128
   int ntile = 0;          // tiles per side
   int ntiles_total = 0;   // ntile diagonal + ntile(ntile-1)/2 off-diagonal
   int64_t nsplit = 0;     // row ranges
   int64_t rows_per_split = 0;
   size_t partial_doubles() const { return (size_t)nsplit * ntiles_total * T * T; }
 };
-// ctas_per_sm: target number of Gram CTAs per SM (an autotuned knob).
-GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm = 4);
+// ctas_per_sm: most Gram CTAs per SM (an autotuned knob); row_unit: the ranges'
+// row counts are multiples of it.
+GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm = 4, int row_unit = 4);
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g,
                           double* partial, cudaStream_t s);
 cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw,
@@ -39,9 +40,11 @@ cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double*
 // Q = A Rinv for upper-triangular Rinv (Algorithm CQR step 3).
 // Small-n path (n <= 256): one row per lane, warps own column groups.
 int qform_group_width(int n);  // columns per group (RP_GROUPS groups), 0 if n > 256
+constexpr int QFORM_PANEL = 32;  // rows of a Q-form panel
 constexpr int RP_GROUPS = 16;  // column groups of the packed R^-1 (the Q-form's NGROUP; checked at run time)
 size_t rpack_doubles(int n);
-// Rp[g][k][c] = Rinv(k, g*w + c) for k <= g*w + c, else 0; Rinv = Y^T.
+// Rp[g][k][c] = Rinv(k, j) for k <= j = g*w + c - lead, else 0, with lead =
+// w ceil(n/w) - n (c < w rounded up to even); Rinv = Y^T.
 cudaError_t pack_rinv_from_lower(const double* Y, int64_t ldy, int n, double* Rp, cudaStream_t s);
 // Same from an upper-triangular Rinv (strictly lower part ignored).
 cudaError_t pack_rinv_from_upper(const double* Rinv, int64_t ld, int n, double* Rp, cudaStream_t s);

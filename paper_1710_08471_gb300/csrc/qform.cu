@@ -4,49 +4,56 @@
 // chip, so Q1 is not read back from memory for the Gram).
 //
 // R^-1 is upper triangular, so column j of Q needs only k <= j. One lane
-// owns one row of a 32-row panel; a warp owns a group of w = n/16 adjacent
-// columns, so every lane of a warp runs the same k range and no FP64 lane is
-// spent on the zero triangle. Warp v takes column groups v and 15 - v, which
-// gives all eight warps the same amount of work. R^-1 is pre-packed per group
-// ([group][k][c], contiguous in c) and read through the read-only path as a
-// warp-wide broadcast; the A panel is staged in shared memory as [k][row],
-// which makes both the global loads and the shared loads conflict-free.
+// owns one row of a 32-row panel; a warp owns groups of w = ceil(n / 16)
+// adjacent columns, so every lane of a warp runs the same k range and no FP64
+// lane is spent on the zero triangle. The ng = ceil(n / w) groups end at column
+// n - 1, so the columns a ragged n lacks are missing from the first group,
+// whose k range is the shortest, and not from the last, whose is the longest.
+// Warp v takes groups v and ng - 1 - v, which evens out the warps' work. (Groups
+// of a power of two from column 0 on, as before: at n = 100 the busiest warp
+// had 1.5 times the mean.) R^-1 is pre-packed per group ([group][k][c],
+// c padded to an even count for 16-byte loads) and read through the read-only
+// path as a warp-wide broadcast; the A panel is staged in shared memory as
+// [k][row], which makes both the global loads and the shared loads
+// conflict-free.
 #include <algorithm>
 
+#include "gram_pairs.cuh"
 #include "kernels.h"
 
 namespace cqr2 {
 namespace {
 
-constexpr int PANEL = 32;   // rows per panel (one per lane)
+constexpr int PANEL = QFORM_PANEL;  // rows per panel (one per lane)
 constexpr int NGROUP = 16;  // column groups
 constexpr int QT = 256;     // threads per CTA
 
+__host__ __device__ constexpr int pitch_of(int w) { return w + (w & 1); }
+// Columns missing from the first group.
+__host__ __device__ constexpr int lead_of(int n, int w) { return (n + w - 1) / w * w - n; }
+
 __global__ void k_pack_rinv(const double* __restrict__ X, int64_t ldx, int n, int w, bool from_lower,
                             double* __restrict__ Rp) {
-  const int64_t total = (int64_t)NGROUP * n * w;
+  const int wp = pitch_of(w), lead = lead_of(n, w);
+  const int64_t total = (int64_t)NGROUP * n * wp;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % w);
-    const int k = (int)((e / w) % n);
-    const int g = (int)(e / ((int64_t)w * n));
-    const int col = g * w + c;
+    const int c = (int)(e % wp);
+    const int k = (int)((e / wp) % n);
+    const int g = (int)(e / ((int64_t)wp * n));
+    const int col = g * w + c - lead;
     double v = 0.0;
-    if (col < n && k <= col) v = from_lower ? X[col + (int64_t)k * ldx] : X[k + (int64_t)col * ldx];
+    if (c < w && col >= 0 && col < n && k <= col) v = from_lower ? X[col + (int64_t)k * ldx] : X[k + (int64_t)col * ldx];
     Rp[e] = v;
   }
 }
 
 template <int W>
 __device__ __forceinline__ void load_w(const double* __restrict__ p, double (&r)[W]) {
-  if constexpr (W >= 2) {
 #pragma unroll
-    for (int c = 0; c < W; c += 2) {
-      const double2 v = __ldg(reinterpret_cast<const double2*>(p + c));
-      r[c] = v.x;
-      r[c + 1] = v.y;
-    }
-  } else {
-    r[0] = __ldg(p);
+  for (int c = 0; c < W; c += 2) {
+    const double2 v = __ldg(reinterpret_cast<const double2*>(p + c));
+    r[c] = v.x;
+    if (c + 1 < W) r[c + 1] = v.y;
   }
 }
 
@@ -54,25 +61,26 @@ __device__ __forceinline__ void load_w(const double* __restrict__ p, double (&r)
 template <int W>
 __device__ __forceinline__ void qform_group(const double* As, int lane, int n, int g,
                                             const double* __restrict__ Rp, double (&acc)[W]) {
-  const int c0 = g * W;
-  const double* rp = Rp + (int64_t)g * n * W;
+  constexpr int WP = pitch_of(W);
+  const int c0 = g * W - lead_of(n, W);  // negative for a ragged first group
+  const double* rp = Rp + (int64_t)g * n * WP;
 #pragma unroll
   for (int c = 0; c < W; ++c) acc[c] = 0.0;
 #pragma unroll 4
   for (int k = 0; k < c0; ++k) {
     const double a = As[k * PANEL + lane];
     double r[W];
-    load_w<W>(rp + (int64_t)k * W, r);
+    load_w<W>(rp + (int64_t)k * WP, r);
 #pragma unroll
     for (int c = 0; c < W; ++c) acc[c] = fma(a, r[c], acc[c]);
   }
 #pragma unroll
   for (int kk = 0; kk < W; ++kk) {
     const int k = c0 + kk;
-    if (k < n) {
+    if (k >= 0) {
       const double a = As[k * PANEL + lane];
       double r[W];
-      load_w<W>(rp + (int64_t)k * W, r);
+      load_w<W>(rp + (int64_t)k * WP, r);
 #pragma unroll
       for (int c = kk; c < W; ++c) acc[c] = fma(a, r[c], acc[c]);
     }
@@ -95,6 +103,7 @@ __global__ void __launch_bounds__(QT) k_qform_small(const double* A, int64_t lda
                                                     int64_t npanels) {
   extern __shared__ double As[];  // [n][PANEL]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ng = (n + W - 1) / W, lead = lead_of(n, W);
   for (int64_t panel = blockIdx.x; panel < npanels; panel += gridDim.x) {
     const int64_t row0 = panel * PANEL;
     stage_panel(A, lda, m, n, row0, As);
@@ -102,61 +111,35 @@ __global__ void __launch_bounds__(QT) k_qform_small(const double* A, int64_t lda
     const int64_t row = row0 + lane;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-      const int g = half ? (NGROUP - 1 - warp) : warp;
-      if (g * W >= n) continue;
+      const int g = half ? ng - 1 - warp : warp;
+      if (half ? g <= warp : 2 * warp > ng - 1) continue;
       double acc[W];
       qform_group<W>(As, lane, n, g, Rp, acc);
       if (row < m) {
 #pragma unroll
         for (int c = 0; c < W; ++c)
-          if (g * W + c < n) Q[row + (int64_t)(g * W + c) * ldq] = acc[c];
+          if (g * W + c >= lead) Q[row + (int64_t)(g * W + c - lead) * ldq] = acc[c];
       }
     }
     __syncthreads();
   }
 }
 
-// Fused Q-form + Gram for n <= T (one diagonal Gram tile of width T). The
-// Gram part is the flattened-upper-pair scheme of the Gram kernel, reading
-// the freshly formed Q panel from shared memory ([row][col], padded).
-template <int W, int T>
+// Fused Q-form + Gram for n <= 128 (one diagonal Gram tile), MAXS >=
+// gram_slots(n). The Gram part reads the freshly formed Q panel from shared
+// memory ([row][col], odd pitch).
+template <int W, int MAXS>
 __global__ void __launch_bounds__(QT) k_qform_gram_small(const double* A, int64_t lda, int64_t m, int n,
                                                          const double* __restrict__ Rp, double* Q, int64_t ldq,
-                                                         int64_t rows_per_split, int ntiles_total,
-                                                         double* __restrict__ partial) {
-  constexpr int LDQ = T + 1;
-  constexpr int P = T * (T + 1) / 2;
-  constexpr int S = (P + QT - 1) / QT;
+                                                         int64_t rows_per_split, int T, double* __restrict__ partial) {
+  static_assert(QT == GRAM_NT, "the pair list is dealt to this block's threads");
   extern __shared__ double smem[];
+  const int pitch = n | 1, ng = (n + W - 1) / W, lead = lead_of(n, W);
   double* As = smem;                       // [n][PANEL]
-  double* Qs = smem + (size_t)T * PANEL;   // [PANEL][LDQ]
+  double* Qs = smem + (size_t)n * PANEL;   // [PANEL][pitch]
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-
-  int oi[S], oj[S];
-  bool last_ok = true;
-  {
-    int i = 0, start = 0;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-      int p = t + s * QT;
-      if (p >= P) {
-        p = P - 1;
-        last_ok = false;
-      }
-      while (p >= start + (T - i)) {
-        start += T - i;
-        ++i;
-      }
-      oi[s] = i;
-      oj[s] = i + (p - start);
-    }
-  }
-  double gacc[S];
-#pragma unroll
-  for (int s = 0; s < S; ++s) gacc[s] = 0.0;
-  // Columns n..T-1 of the staged Q panel stay zero.
-  for (int e = t; e < PANEL * LDQ; e += QT) Qs[e] = 0.0;
-  __syncthreads();
+  GramPairs<MAXS> pairs;
+  pairs.init(t, n);
 
   const int64_t r_begin = (int64_t)blockIdx.x * rows_per_split;
   const int64_t r_end = min(m, r_begin + rows_per_split);
@@ -166,32 +149,24 @@ __global__ void __launch_bounds__(QT) k_qform_gram_small(const double* A, int64_
     const int64_t row = row0 + lane;
 #pragma unroll 1
     for (int half = 0; half < 2; ++half) {
-      const int g = half ? (NGROUP - 1 - warp) : warp;
-      if (g * W >= n) continue;
+      const int g = half ? ng - 1 - warp : warp;
+      if (half ? g <= warp : 2 * warp > ng - 1) continue;
       double acc[W];
       qform_group<W>(As, lane, n, g, Rp, acc);
 #pragma unroll
       for (int c = 0; c < W; ++c) {
-        const int col = g * W + c;
-        if (col < n) {
-          Qs[lane * LDQ + col] = acc[c];
+        const int col = g * W + c - lead;
+        if (col >= 0) {
+          Qs[lane * pitch + col] = acc[c];
           if (row < r_end) Q[row + (int64_t)col * ldq] = acc[c];
         }
       }
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < PANEL; ++kk) {
-      const double* qrow = Qs + kk * LDQ;
-#pragma unroll
-      for (int s = 0; s < S; ++s) gacc[s] = fma(qrow[oi[s]], qrow[oj[s]], gacc[s]);
-    }
+    pairs.add(Qs, pitch, PANEL);
     __syncthreads();
   }
-  double* out = partial + (int64_t)blockIdx.x * ntiles_total * (int64_t)(T * T);
-#pragma unroll
-  for (int s = 0; s < S; ++s)
-    if (s < S - 1 || last_ok) out[oi[s] + oj[s] * T] = gacc[s];
+  pairs.store(partial + (int64_t)blockIdx.x * (T * T), T);
 }
 
 int sm_count() {
@@ -206,7 +181,8 @@ cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const d
                          cudaStream_t s) {
   const size_t sm = (size_t)n * PANEL * sizeof(double);
   auto kern = k_qform_small<W>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(16 * W * PANEL * sizeof(double)));  // of the widest matrix
   if (e != cudaSuccess) return e;
   const int64_t npanels = ceil_div(m, PANEL);
   int per_sm = 1;
@@ -217,37 +193,33 @@ cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const d
   return cudaGetLastError();
 }
 
-template <int W, int T>
+template <int W, int MAXS>
 cudaError_t launch_fused(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q, int64_t ldq,
                          const GramGeom& g, double* partial, cudaStream_t s) {
-  const size_t sm = ((size_t)T * PANEL + (size_t)PANEL * (T + 1)) * sizeof(double);
-  auto kern = k_qform_gram_small<W, T>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  static_assert(MAXS >= gram_slots(16 * W > 128 ? 128 : 16 * W), "slots of the widest matrix of this group width");
+  const size_t sm = ((size_t)n * PANEL + (size_t)PANEL * (n | 1)) * sizeof(double);
+  auto kern = k_qform_gram_small<W, MAXS>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)((128 + 129) * PANEL * sizeof(double)));
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)g.nsplit, QT, sm, s>>>(A, lda, m, n, Rp, Q, ldq, g.rows_per_split, g.ntiles_total, partial);
+  kern<<<(unsigned)g.nsplit, QT, sm, s>>>(A, lda, m, n, Rp, Q, ldq, g.rows_per_split, g.T, partial);
   count_launch();
   return cudaGetLastError();
 }
 
 }  // namespace
 
-int qform_group_width(int n) {
-  if (n > 256) return 0;
-  const int w = (int)ceil_div(n, NGROUP);
-  int p = 1;
-  while (p < w) p *= 2;
-  return p;
-}
+int qform_group_width(int n) { return n > 256 ? 0 : (int)ceil_div(n, NGROUP); }
 
 size_t rpack_doubles(int n) {
   const int w = qform_group_width(n);
-  return (size_t)NGROUP * n * (w ? w : 0);
+  return (size_t)NGROUP * n * (w ? pitch_of(w) : 0);
 }
 
 static cudaError_t pack(const double* X, int64_t ldx, int n, bool lower, double* Rp, cudaStream_t s) {
   const int w = qform_group_width(n);
   if (!w) return cudaErrorInvalidValue;
-  const int64_t total = (int64_t)NGROUP * n * w;
+  const int64_t total = (int64_t)rpack_doubles(n);
   const int grid = (int)std::min<int64_t>(ceil_div(total, 256), 4096);
   k_pack_rinv<<<grid, 256, 0, s>>>(X, ldx, n, w, lower, Rp);
   count_launch();
@@ -267,8 +239,19 @@ cudaError_t qform_small(const double* A, int64_t lda, int64_t m, int n, const do
   switch (qform_group_width(n)) {
     case 1: return launch_qform<1>(A, lda, m, n, Rp, Q, ldq, s);
     case 2: return launch_qform<2>(A, lda, m, n, Rp, Q, ldq, s);
+    case 3: return launch_qform<3>(A, lda, m, n, Rp, Q, ldq, s);
     case 4: return launch_qform<4>(A, lda, m, n, Rp, Q, ldq, s);
+    case 5: return launch_qform<5>(A, lda, m, n, Rp, Q, ldq, s);
+    case 6: return launch_qform<6>(A, lda, m, n, Rp, Q, ldq, s);
+    case 7: return launch_qform<7>(A, lda, m, n, Rp, Q, ldq, s);
     case 8: return launch_qform<8>(A, lda, m, n, Rp, Q, ldq, s);
+    case 9: return launch_qform<9>(A, lda, m, n, Rp, Q, ldq, s);
+    case 10: return launch_qform<10>(A, lda, m, n, Rp, Q, ldq, s);
+    case 11: return launch_qform<11>(A, lda, m, n, Rp, Q, ldq, s);
+    case 12: return launch_qform<12>(A, lda, m, n, Rp, Q, ldq, s);
+    case 13: return launch_qform<13>(A, lda, m, n, Rp, Q, ldq, s);
+    case 14: return launch_qform<14>(A, lda, m, n, Rp, Q, ldq, s);
+    case 15: return launch_qform<15>(A, lda, m, n, Rp, Q, ldq, s);
     case 16: return launch_qform<16>(A, lda, m, n, Rp, Q, ldq, s);
     default: return cudaErrorInvalidValue;
   }
@@ -279,17 +262,16 @@ bool qform_gram_fusable(int n) { return n >= 1 && n <= 128; }
 cudaError_t qform_gram_small(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q,
                              int64_t ldq, const GramGeom& g, double* partial, cudaStream_t s) {
   if (!qform_gram_fusable(n) || g.ntile != 1 || g.T < n) return cudaErrorInvalidValue;
-  const int w = qform_group_width(n);
-  switch (g.T) {
-    case 32:
-      if (w == 1) return launch_fused<1, 32>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
-      return launch_fused<2, 32>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
-    case 64:
-      return launch_fused<4, 64>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
-    case 128:
-      return launch_fused<8, 128>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
-    default:
-      return cudaErrorInvalidValue;
+  switch (qform_group_width(n)) {
+    case 1: return launch_fused<1, 8>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 2: return launch_fused<2, 8>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 3: return launch_fused<3, 8>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 4: return launch_fused<4, 16>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 5: return launch_fused<5, 16>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 6: return launch_fused<6, 24>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 7: return launch_fused<7, 33>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    case 8: return launch_fused<8, 33>(A, lda, m, n, Rp, Q, ldq, g, partial, s);
+    default: return cudaErrorInvalidValue;
   }
 }
 
