@@ -22,18 +22,32 @@ namespace cqr2 {
 namespace {
 
 constexpr int BT = 256;   // threads
-constexpr int BNMAX = 64; // largest n
-constexpr int BLD = BNMAX + 1;
 constexpr int BPANEL = 32;
-constexpr int BP = BNMAX * (BNMAX + 1) / 2;  // 2080 upper pairs
-constexpr int BS = (BP + BT - 1) / BT;       // 9 slots per thread
 
+// Two sizes of the kernel, n <= 32 and n <= 64. A CTA alone leaves the FP64
+// pipe idle during its serial parts (the two n-step CholInvs, panel loads and
+// barriers). The small size's shared memory (35 KB) and registers let three
+// CTAs share an SM and fill one another's gaps; the large one's 117 KB allow
+// one. 1024 problems of 4096 x 32: 20.0 -> 17.7 ms (14.8 at the pipe's peak; a
+// sixth of the SMs have no seventh problem).
+template <int N_>
+struct SmallCfg {
+  static constexpr int N = N_;                    // largest n
+  static constexpr int LD = N + 1;
+  static constexpr int S = (N * (N + 1) / 2 + BT - 1) / BT;  // slots of upper pairs per thread (3 or 9)
+  static constexpr int PF = BPANEL * N / BT;      // panel entries per thread (4 or 8)
+  static constexpr int NQ = N / 8;                // columns per warp (4 or 8)
+  static constexpr int CTAS = N <= 32 ? 3 : 1;    // per SM
+};
+
+template <int N>
 struct SmallSmem {
-  double S[BNMAX * BLD];   // W, then L (column-major, lower), S(i,j) = S[j*BLD + i]
-  double T[BNMAX * BLD];   // Y = L^-1 (lower)
-  double R1[BNMAX * BLD];  // R1 = L1^T (upper) kept for R = R2 R1
-  double P[BPANEL * BLD];  // row panel of A or Q1, [row][col]
-  double rd[BNMAX];        // reciprocals of L's diagonal
+  static constexpr int LD = SmallCfg<N>::LD;
+  double S[N * LD];       // W, then L (column-major, lower), S(i,j) = S[j*LD + i]
+  double T[N * LD];       // Y = L^-1 (lower)
+  double R1[N * LD];      // R1 = L1^T (upper) kept for R = R2 R1
+  double P[BPANEL * LD];  // row panel of A or Q1, [row][col]
+  double rd[N];           // reciprocals of L's diagonal
   int fail_pivot;
 };
 
@@ -42,7 +56,7 @@ struct SmallSmem {
 // this n is skipped by the whole warp: the FP64 pipe issues a warp
 // instruction at full cost whatever its lane mask or predicate, so the
 // branch sits outside the row loop and idle slots issue nothing.
-template <int NS>
+template <int BLD, int NS>
 __device__ __forceinline__ void gram_panel_ns(const double* __restrict__ Pn, const int* oi, const int* oj,
                                               const bool* wact, double* acc) {
 #pragma unroll
@@ -56,45 +70,56 @@ __device__ __forceinline__ void gram_panel_ns(const double* __restrict__ Pn, con
   }
 }
 
+template <int N>
 __device__ __forceinline__ void gram_panel(int nslots, const double* Pn, const int* oi, const int* oj,
                                            const bool* wact, double* acc) {
-  switch (nslots) {
-    case 1: gram_panel_ns<1>(Pn, oi, oj, wact, acc); break;
-    case 2: gram_panel_ns<2>(Pn, oi, oj, wact, acc); break;
-    case 3: gram_panel_ns<3>(Pn, oi, oj, wact, acc); break;
-    case 4: gram_panel_ns<4>(Pn, oi, oj, wact, acc); break;
-    case 5: gram_panel_ns<5>(Pn, oi, oj, wact, acc); break;
-    case 6: gram_panel_ns<6>(Pn, oi, oj, wact, acc); break;
-    case 7: gram_panel_ns<7>(Pn, oi, oj, wact, acc); break;
-    case 8: gram_panel_ns<8>(Pn, oi, oj, wact, acc); break;
-    default: gram_panel_ns<BS>(Pn, oi, oj, wact, acc); break;
+  constexpr int BLD = SmallCfg<N>::LD, BS = SmallCfg<N>::S;
+  if constexpr (BS <= 3) {
+    switch (nslots) {
+      case 1: gram_panel_ns<BLD, 1>(Pn, oi, oj, wact, acc); break;
+      case 2: gram_panel_ns<BLD, 2>(Pn, oi, oj, wact, acc); break;
+      default: gram_panel_ns<BLD, BS>(Pn, oi, oj, wact, acc); break;
+    }
+  } else {
+    switch (nslots) {
+      case 3: gram_panel_ns<BLD, 3>(Pn, oi, oj, wact, acc); break;
+      case 4: gram_panel_ns<BLD, 4>(Pn, oi, oj, wact, acc); break;
+      case 5: gram_panel_ns<BLD, 5>(Pn, oi, oj, wact, acc); break;
+      case 6: gram_panel_ns<BLD, 6>(Pn, oi, oj, wact, acc); break;
+      case 7: gram_panel_ns<BLD, 7>(Pn, oi, oj, wact, acc); break;
+      case 8: gram_panel_ns<BLD, 8>(Pn, oi, oj, wact, acc); break;
+      default: gram_panel_ns<BLD, BS>(Pn, oi, oj, wact, acc); break;
+    }
   }
 }
 
 // Register prefetch of a 32-row panel (all n columns): thread t holds the
 // elements e = t + BT i of the panel, e = r + 32 c. Issued before the current
 // panel's arithmetic, so the global load latency overlaps it.
-constexpr int PF = BPANEL * BNMAX / BT;  // 8
+template <int N>
 __device__ __forceinline__ void panel_load(const double* X, int64_t ldx, int64_t m, int n, int64_t r0, double* pf) {
 #pragma unroll
-  for (int i = 0; i < PF; ++i) {
+  for (int i = 0; i < SmallCfg<N>::PF; ++i) {
     const int e = threadIdx.x + BT * i;
     const int r = e % BPANEL, c = e / BPANEL;
     pf[i] = (c < n && r0 + r < m) ? X[r0 + r + (int64_t)c * ldx] : 0.0;
   }
 }
+template <int N>
 __device__ __forceinline__ void panel_store(const double* pf, int n, double* P) {
 #pragma unroll
-  for (int i = 0; i < PF; ++i) {
+  for (int i = 0; i < SmallCfg<N>::PF; ++i) {
     const int e = threadIdx.x + BT * i;
     const int r = e % BPANEL, c = e / BPANEL;
-    if (c < n) P[r * BLD + c] = pf[i];
+    if (c < n) P[r * SmallCfg<N>::LD + c] = pf[i];
   }
 }
 
 // Right-looking Cholesky of S (n x n, lower) and inverse into T; returns the
 // first bad pivot index or -1. All threads participate.
-__device__ int cholinv_smem(SmallSmem& sm, int n) {
+template <int N>
+__device__ int cholinv_smem(SmallSmem<N>& sm, int n) {
+  constexpr int BLD = SmallCfg<N>::LD;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
   if (t == 0) sm.fail_pivot = -1;
   for (int e = t; e < n * n; e += BT) {
@@ -134,10 +159,13 @@ __device__ int cholinv_smem(SmallSmem& sm, int n) {
   return sm.fail_pivot;
 }
 
-__global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem* __restrict__ probs, int count,
-                                                           int* __restrict__ next, BatchStatus* __restrict__ status) {
+template <int N>
+__global__ void __launch_bounds__(BT, SmallCfg<N>::CTAS)
+    k_cqr2_small_batched(const BatchProblem* __restrict__ probs, int count, int* __restrict__ next,
+                         BatchStatus* __restrict__ status) {
+  constexpr int BLD = SmallCfg<N>::LD, BS = SmallCfg<N>::S, PF = SmallCfg<N>::PF, NQ = SmallCfg<N>::NQ;
   extern __shared__ double smem_raw[];
-  SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
+  SmallSmem<N>& sm = *reinterpret_cast<SmallSmem<N>*>(smem_raw);
   __shared__ int s_job;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   for (;;) {
@@ -180,12 +208,12 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
       if (pass == 1) {
         // W1 = A^T A
         double pf[PF];
-        panel_load(X, ldx, m, n, 0, pf);
+        panel_load<N>(X, ldx, m, n, 0, pf);
         for (int64_t r0 = 0; r0 < m; r0 += BPANEL) {
-          panel_store(pf, n, sm.P);
+          panel_store<N>(pf, n, sm.P);
           __syncthreads();
-          if (r0 + BPANEL < m) panel_load(X, ldx, m, n, r0 + BPANEL, pf);
-          gram_panel(nslots, sm.P, oi, oj, wact, acc);
+          if (r0 + BPANEL < m) panel_load<N>(X, ldx, m, n, r0 + BPANEL, pf);
+          gram_panel<N>(nslots, sm.P, oi, oj, wact, acc);
           __syncthreads();
         }
       }
@@ -202,7 +230,7 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
           }
         __syncthreads();
       }
-      const int piv = cholinv_smem(sm, n);
+      const int piv = cholinv_smem<N>(sm, n);
       if (piv >= 0 && fail_pass == 0) {
         fail_pass = pass;
         fail_pivot = piv;
@@ -222,23 +250,24 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
       for (int s = 0; s < BS; ++s) gacc[s] = 0.0;
       // pass 2 of a least-squares problem: c = Q^T b, lane = row, per column j
       const bool with_c = pass == 2 && pb.b != nullptr;
-      double cacc[BNMAX / 8];
+      double cacc[NQ];
 #pragma unroll
-      for (int q = 0; q < BNMAX / 8; ++q) cacc[q] = 0.0;
+      for (int q = 0; q < NQ; ++q) cacc[q] = 0.0;
       double pf[PF];
-      panel_load(X, ldx, m, n, 0, pf);
+      panel_load<N>(X, ldx, m, n, 0, pf);
       for (int64_t r0 = 0; r0 < m; r0 += BPANEL) {
-        panel_store(pf, n, sm.P);
+        panel_store<N>(pf, n, sm.P);
         __syncthreads();
         // The next panel's loads go out now. In pass 2, X is Q itself: the
         // next panel's rows are read before this iteration writes (only) the
         // current panel's rows.
-        if (r0 + BPANEL < m) panel_load(X, ldx, m, n, r0 + BPANEL, pf);
-        // each warp owns columns j = warp, warp+8, ...; lane owns row r0+lane
-        double qv[BNMAX / 8];
+        if (r0 + BPANEL < m) panel_load<N>(X, ldx, m, n, r0 + BPANEL, pf);
+        // each warp owns a column of every eight, in a snake (a column's work is
+        // its index plus one: the sums are equal); lane owns row r0+lane
+        double qv[NQ];
 #pragma unroll
-        for (int q = 0; q < BNMAX / 8; ++q) {
-          const int j = warp + 8 * q;
+        for (int q = 0; q < NQ; ++q) {
+          const int j = 8 * q + ((q & 1) ? 7 - warp : warp);
           double a = 0.0;
           if (j < n) {
             for (int k = 0; k <= j; ++k) a = fma(sm.P[lane * BLD + k], sm.T[k * BLD + j], a);
@@ -248,8 +277,8 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
         __syncthreads();  // everyone has read the panel
         const double bv = (with_c && r0 + lane < m) ? pb.b[r0 + lane] : 0.0;
 #pragma unroll
-        for (int q = 0; q < BNMAX / 8; ++q) {
-          const int j = warp + 8 * q;
+        for (int q = 0; q < NQ; ++q) {
+          const int j = 8 * q + ((q & 1) ? 7 - warp : warp);
           if (j < n) {
             sm.P[lane * BLD + j] = qv[q];
             if (r0 + lane < m) pb.Q[r0 + lane + (int64_t)j * pb.ldq] = qv[q];
@@ -257,17 +286,17 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
           }
         }
         __syncthreads();
-        if (pass == 1) gram_panel(nslots, sm.P, oi, oj, wact, gacc);
+        if (pass == 1) gram_panel<N>(nslots, sm.P, oi, oj, wact, gacc);
         __syncthreads();
       }
       if (with_c) {
         // c_j = sum over lanes (fixed xor tree), kept in sm.P[j]
 #pragma unroll
-        for (int q = 0; q < BNMAX / 8; ++q) {
+        for (int q = 0; q < NQ; ++q) {
           double v = cacc[q];
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-          const int j = warp + 8 * q;
+          const int j = 8 * q + ((q & 1) ? 7 - warp : warp);
           if (lane == 0 && j < n) sm.P[j] = v;
         }
         __syncthreads();
@@ -319,21 +348,27 @@ __global__ void __launch_bounds__(BT, 1) k_cqr2_small_batched(const BatchProblem
 
 }  // namespace
 
-size_t batched_small_smem() { return sizeof(SmallSmem); }
-
-cudaError_t cqr2_small_batched(const BatchProblem* probs, int count, int* next, BatchStatus* status, cudaStream_t s) {
-  const size_t sm = sizeof(SmallSmem);
-  cudaError_t e = cudaFuncSetAttribute(k_cqr2_small_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+template <int N>
+static cudaError_t launch_small(const BatchProblem* probs, int count, int* next, BatchStatus* status, cudaStream_t s) {
+  const size_t sm = sizeof(SmallSmem<N>);
+  auto kern = k_cqr2_small_batched<N>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 148, per = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cqr2_small_batched, BT, sm);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, BT, sm);
   const int grid = std::max(1, std::min(count, sms * std::max(1, per)));
   if ((e = cudaMemsetAsync(next, 0, sizeof(int), s)) != cudaSuccess) return e;
-  k_cqr2_small_batched<<<grid, BT, sm, s>>>(probs, count, next, status);
+  kern<<<grid, BT, sm, s>>>(probs, count, next, status);
   count_launch();
   return cudaGetLastError();
+}
+
+cudaError_t cqr2_small_batched(const BatchProblem* probs, int count, int* next, BatchStatus* status, bool narrow,
+                               cudaStream_t s) {
+  return narrow ? launch_small<BATCH_NARROW_N>(probs, count, next, status, s)
+                : launch_small<BATCH_SMALL_MAX_N>(probs, count, next, status, s);
 }
 
 }  // namespace cqr2

@@ -194,11 +194,11 @@ struct BatchStatus {
   int failed_pivot;  // -1 = none
 };
 constexpr int BATCH_SMALL_MAX_N = 64;
+constexpr int BATCH_NARROW_N = 32;  // problems up to here take the kernel's small size
 // Enqueue a copy of a plan's device status word (outcome of its last call).
 cudaError_t plan_status_copy(struct ::cqr2_plan_st* p, DevStatus* dst, cudaStream_t s);
-size_t batched_small_smem();
-// Persistent grouped kernel: every problem (n <= 64) factored by one CTA.
-cudaError_t cqr2_small_batched(const BatchProblem* probs, int count, int* next, BatchStatus* status,
+// Persistent grouped kernel: every problem (n <= 64; narrow: n <= 32) factored by one CTA.
+cudaError_t cqr2_small_batched(const BatchProblem* probs, int count, int* next, BatchStatus* status, bool narrow,
                                cudaStream_t s);
 
 // ---------------------------------------------------------------- panels
