@@ -29,7 +29,7 @@ constexpr int BPANEL = 32;
 // barriers). The small size's shared memory (35 KB) and registers let three
 // CTAs share an SM and fill one another's gaps; the large one's 117 KB allow
 // one. 1024 problems of 4096 x 32: 20.0 -> 17.7 ms (14.8 at the pipe's peak; a
-// sixth of the SMs have no seventh problem).
+// quarter of the SMs have no seventh problem).
 template <int N_>
 struct SmallCfg {
   static constexpr int N = N_;                    // largest n

@@ -128,8 +128,6 @@ constexpr int OZAKI_MAX_N = 16384;
 struct OzGeom {
   int64_t mp = 0;            // m rounded up to 64
   int np = 0;                // n rounded up to 64
-  int ntile_j = 0;           // Gram: 64-column tiles
-  int ntiles = 0;            // Gram tiles (128 x 64) touching the upper triangle
   int64_t rows_per_split = 0;
   int nsplit = 0;
 };
