@@ -188,4 +188,41 @@ OZ_HD double oz_xy_to_double_fast(long long X, long long Y, int E) {
   return oz_bits_to_double(bits | (neg ? 1ull << 63 : 0ull));
 }
 
+// The same for a group of outputs with one shift: T 2^-(24-s) = X 2^s + Y
+// 2^-(24-s) fits 62 bits for every output of the group when s = min(24, 62 -
+// (bits of the largest |X|)), and what falls off Y (rounded) is then below
+// 2^-61 of the group's largest |T|. The hardware converts that integer with one
+// correct rounding (one FP64 operation), and the exponent is added to its bits:
+// about a quarter of the instructions of the normalising sequence above, which
+// was most of the Q-form's epilogue.
+// h: the OR over the group of oz_high_bits(X).
+OZ_HD unsigned oz_high_bits(long long X) {
+  const int hi = (int)(X >> 32);
+  return (unsigned)(hi ^ (hi >> 31));
+}
+OZ_HD int oz_group_shift(unsigned h) {
+#if defined(__CUDA_ARCH__)
+  const int lz = __clz((int)h);
+#else
+  const int lz = h ? __builtin_clz(h) : 32;
+#endif
+  return lz - 2 < 24 ? lz - 2 : 24;
+}
+OZ_HD double oz_xy_to_double_group(long long X, long long Y, int s, int E) {
+  const int sh = 24 - s;
+  const long long Z = (long long)((unsigned long long)X << s) + ((Y + ((1ll << sh) >> 1)) >> sh);
+#if defined(__CUDA_ARCH__)
+  const double d = __ll2double_rn(Z);
+#else
+  const double d = (double)Z;
+#endif
+  const unsigned long long b = (unsigned long long)oz_double_bits(d);
+  const int e = E + sh, ex = (int)((b >> 52) & 0x7FF), biased = ex + e;
+  if (ex == 0 || (unsigned)(biased - 1) >= 2046u) {  // zero, or a result outside the normal range
+    if (Z == 0) return 0.0;
+    return OZ_XY_COLD(X, Y, E);
+  }
+  return oz_bits_to_double(b + ((unsigned long long)(long long)e << 52));
+}
+
 }  // namespace cqr2

@@ -908,6 +908,11 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
         const int ea2 = MODE == OZ_GRAM ? p.eA[row] : ea;
         double* out = MODE == OZ_GRAM ? p.out + (int64_t)w.split * p.n * p.n : p.out;
         const int64_t ld = MODE == OZ_GRAM ? p.n : p.ldo;
+        unsigned h = 0;  // Q-form: one shift for this thread's outputs
+        if (MODE == OZ_QFORM)
+#pragma unroll
+          for (int cc = 0; cc < CPT; ++cc) h |= oz_high_bits(X[cc]);
+        const int shift = oz_group_shift(h);
 #pragma unroll
         for (int cc = 0; cc < CPT; ++cc) {
           const int64_t col = w.j0 + cs * CPT + cc;
@@ -918,7 +923,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
             const double v = (ea2 >= EXP_NONFINITE || e2 >= EXP_NONFINITE)
                                  ? __longlong_as_double(0x7FF8000000000000ll)
                              : MODE == OZ_GRAM ? oz_xy_to_double(X[cc], Y[cc], ea2 + e2 - 14 - 48)
-                                               : oz_xy_to_double_fast(X[cc], Y[cc], ea2 + e2 - 14 - 48);
+                                               : oz_xy_to_double_group(X[cc], Y[cc], shift, ea2 + e2 - 14 - 48);
             out[row + col * ld] = v;
             if (MODE == OZ_QFORM && fuse_cmax) ck[cc < NEB ? cc : 0] = oz_exp_key(v);
           }
