@@ -25,7 +25,7 @@ def _nearest(x):
     try:
         return float(x)  # Fraction to the nearest double, subnormals included
     except OverflowError:
-        return math.copysign(math.inf, x)
+        return math.inf if x > 0 else -math.inf
 
 
 def test_group_conversion(tmp_path):
