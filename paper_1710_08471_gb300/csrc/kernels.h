@@ -131,12 +131,13 @@ struct OzGeom {
   int64_t rows_per_split = 0;
   int nsplit = 0;
 };
-// Four TMA descriptors (CUtensorMap is 128 bytes, 64-byte aligned).
+// TMA descriptors (CUtensorMap is 128 bytes, 64-byte aligned).
 struct OzMaps {
   alignas(64) unsigned char col_a[128];
   alignas(64) unsigned char col_b[128];
   alignas(64) unsigned char col_a_mn[128];  // the column slices as the Q-form's MN-major left operand
   alignas(64) unsigned char rinv_b[128];
+  alignas(64) unsigned char rinv_b_wide[128];  // the same in boxes of 64 columns
 };
 bool ozaki_supported(int n, int S);
 OzGeom ozaki_geometry(int64_t m, int n);
@@ -170,7 +171,7 @@ cudaError_t ozaki_qform(const OzMaps& maps, int64_t m, int n, int S, const int* 
 // exceeds 16 (or, with keep, when *gate is 7 already), else to 6.
 cudaError_t ozaki_route(const int* cexp, const double* W, int64_t ldw, int n, int64_t m, int* gate, bool keep,
                         cudaStream_t s);
-constexpr int OZAKI_FUSED_COLMAX_MAX_N = 1024;
+constexpr int OZAKI_FUSED_COLMAX_MAX_N = 512;
 // Column exponents from column maxima (the second half of ozaki_colmax).
 cudaError_t ozaki_exps(const unsigned long long* colmax, int n, int* cexp, cudaStream_t s);
 

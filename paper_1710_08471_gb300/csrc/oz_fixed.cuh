@@ -208,7 +208,10 @@ OZ_HD int oz_group_shift(unsigned h) {
 #endif
   return lz - 2 < 24 ? lz - 2 : 24;
 }
-OZ_HD double oz_xy_to_double_group(long long X, long long Y, int s, int E) {
+// The conversion without its rare cases, so that a kernel can run several side
+// by side without branches; ok is false for zero and for a result outside the
+// normal range, which oz_xy_to_double_group (below) then forms.
+OZ_HD double oz_xy_to_double_group_fast(long long X, long long Y, int s, int E, bool* ok) {
   const int sh = 24 - s;
   const long long Z = (long long)((unsigned long long)X << s) + ((Y + ((1ll << sh) >> 1)) >> sh);
 #if defined(__CUDA_ARCH__)
@@ -217,12 +220,17 @@ OZ_HD double oz_xy_to_double_group(long long X, long long Y, int s, int E) {
   const double d = (double)Z;
 #endif
   const unsigned long long b = (unsigned long long)oz_double_bits(d);
-  const int e = E + sh, ex = (int)((b >> 52) & 0x7FF), biased = ex + e;
-  if (ex == 0 || (unsigned)(biased - 1) >= 2046u) {  // zero, or a result outside the normal range
-    if (Z == 0) return 0.0;
-    return OZ_XY_COLD(X, Y, E);
-  }
+  const int e = E + sh, ex = (int)((b >> 52) & 0x7FF);
+  *ok = ex != 0 && (unsigned)(ex + e - 1) < 2046u;
   return oz_bits_to_double(b + ((unsigned long long)(long long)e << 52));
+}
+OZ_HD double oz_xy_to_double_group(long long X, long long Y, int s, int E) {
+  bool ok;
+  const double v = oz_xy_to_double_group_fast(X, Y, s, E, &ok);
+  if (ok) return v;
+  const int sh = 24 - s;
+  const long long Z = (long long)((unsigned long long)X << s) + ((Y + ((1ll << sh) >> 1)) >> sh);
+  return Z == 0 ? 0.0 : OZ_XY_COLD(X, Y, E);
 }
 
 }  // namespace cqr2

@@ -21,8 +21,8 @@
 // warps move the group sums into two int64 fixed-point accumulators per
 // output (T = X 2^24 + Y, X: groups 0-3, Y: groups 4-6), which stays exact
 // as well. The only roundings are the one of x' and the final conversion to
-// FP64 with integer operations: correctly rounded for the Gram, within one
-// ulp for the Q-form (a shorter sequence; far below its truncation error).
+// FP64: correctly rounded for the Gram (integer operations), within one ulp for
+// the Q-form (a shorter sequence; far below its truncation error).
 //
 // Kernel: persistent, one CTA per SM. BF16 operands in 128-byte swizzled
 // shared memory, loaded by TMA from the column slice planes, stored K-block
@@ -30,9 +30,9 @@
 // (the Q-form's X as an MN-major operand, everything else K-major). Warp 0
 // produces (TMA), warp 1 issues tcgen05.mma (M = 128, one MMA per A slice and
 // K = 16 step covering all its products), the other warps drain the group
-// accumulators. Gram: 128 x 64 tiles, one accumulator buffer; Q-form:
-// 128 x 32 tiles, two. All waits are bounded; a timeout sets the status word
-// and the CTA unwinds.
+// accumulators. Gram: 128 x 64 tiles, one accumulator buffer; Q-form: the same
+// or 128 x 32 tiles with two (oz_qform_shape). All waits are bounded; a timeout
+// sets the status word and the CTA unwinds.
 #include <cuda.h>
 
 #include <algorithm>
@@ -45,7 +45,7 @@ namespace cqr2 {
 namespace {
 
 constexpr int OZ_BK = 64;          // contraction per K-block (128-byte rows)
-constexpr int OZ_QFORM_NA_MAX = 10;  // A ring slots of the Q-form (the Gram keeps 8)
+constexpr int OZ_NA_MAX = 10;      // most A ring slots
 constexpr int OZ_BM = 128;         // tile rows
 constexpr int EXP_NONFINITE = OZ_EXP_NONFINITE;
 constexpr long long WAIT_LIMIT = 1ll << 24;
@@ -236,6 +236,28 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t phase, const Dev
   return false;
 }
 
+// The same by a whole warp in step (every lane gets the same answer from a
+// vote, so the compiler keeps what follows in uniform registers).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* b, uint32_t phase, const DevStatus* st) {
+  const uint32_t addr = smem_u32(b);
+  for (long long i = 0; i < WAIT_LIMIT; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(addr), "r"(phase)
+        : "memory");
+    if (__all_sync(0xffffffffu, ok)) return true;
+    if ((i & 4095) == 4095 && __any_sync(0xffffffffu, *(volatile const int*)&st->status == 5)) return false;
+  }
+  return false;
+}
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+  return e != 0;
+}
+
 // Bounded wait that ignores the status word: after a timeout, the unwinding
 // CTA still waits (up to the limit) for its own copies and MMAs in flight.
 __device__ __forceinline__ bool mbar_wait_drain(uint64_t* b, uint32_t phase) {
@@ -299,13 +321,13 @@ __device__ __forceinline__ uint32_t pair_rank() {
 // MN-major operand (the Q-form's X tile, [k][m] rows of 64 m-values): 128-byte
 // swizzle, 64-element atoms along M 8192 bytes apart (the two TMA boxes), 8-row
 // groups along K 1024 bytes apart; 16 k further is 2048 bytes.
-__device__ __forceinline__ uint64_t sdesc_mn(const void* p) {
-  const uint64_t a = (smem_u32(p) & 0x3FFFF) >> 4;
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t p) {
+  const uint64_t a = (p & 0x3FFFF) >> 4;
   return a | ((uint64_t)(8192 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
 }
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t sdesc(const void* p) {
-  const uint64_t a = (smem_u32(p) & 0x3FFFF) >> 4;
+__device__ __forceinline__ uint64_t sdesc(uint32_t p) {
+  const uint64_t a = (p & 0x3FFFF) >> 4;
   return a | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
 }
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
@@ -339,33 +361,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 
 enum { OZ_GRAM = 0, OZ_QFORM = 1 };
 
-// Tile shapes. The Gram uses 128 x 64 tiles (more operand reuse; the S group
-// accumulators take 64 S <= 448 TMEM columns, one buffer). The Q-form uses
-// 128 x 32 tiles with two accumulator buffers (2 x 32 S <= 448 columns) and
-// 16 epilogue warps, since its epilogue (S conversions to integer and one to
-// FP64 per output) is as long as its MMAs. The epilogue warps may also be
-// split into two groups that take alternate tiles (NGRP = 2); measured on
-// 2^20 x 128 that was slower (1.88 ms against 1.37 ms per Q-form), so both
-// shapes run one group.
+// Tile shapes. 128 x 64 tiles (the Gram, and the Q-form where oz_qform_shape
+// says so) reuse their operands more; the S group accumulators take 64 S <= 448
+// TMEM columns, one buffer. 128 x 32 tiles have two accumulator buffers (2 x 32
+// S <= 448 columns). The Q-form has 16 epilogue warps, since its epilogue (S
+// conversions to integer and one to FP64 per output) is nearly as long as its
+// MMAs. The epilogue warps may also be split into two groups that take
+// alternate tiles (NGRP = 2); measured on 2^20 x 128 that was slower (1.88 ms
+// against 1.37 ms per Q-form), so all shapes run one group.
 constexpr int OZ_GRAM_BN = 64, OZ_GRAM_EPI = 8, OZ_GRAM_GRP = 1;
-constexpr int OZ_QFORM_BN = 32, OZ_QFORM_EPI = 16, OZ_QFORM_GRP = 1;
+constexpr int OZ_QFORM_BN = 32, OZ_QFORM_BN_WIDE = 64, OZ_QFORM_EPI = 16, OZ_QFORM_GRP = 1;
 
-template <int S, int BN, int EPI, int NGRP>
+template <int S, int MODE, int BN, int EPI, int NGRP>
 struct OzCfg {
   static constexpr int NBUF = 2 * S * BN <= 512 ? 2 : 1;         // accumulator buffers in TMEM
   static constexpr int THREADS = 64 + 32 * EPI;                   // producer, MMA, epilogue warps
   static constexpr int A_BYTES = OZ_BM * OZ_BK * 2;               // one A slice tile
   static constexpr int B_BYTES = BN * OZ_BK * 2;                  // one B slice tile
+  // Q-form: column-max keys, for as many columns as the ring leaves room for
+  static constexpr int KEYS = MODE == OZ_QFORM ? 512 : 0;
   // A ring slots: what shared memory leaves beside the B double buffer, the
-  // barriers and (Q-form) the column-max keys, at most 8 (Gram) or 10
-  static constexpr int RESERVED = BN == 32 ? 6200 : 2048, NA_CAP = BN == 32 ? OZ_QFORM_NA_MAX : 8;
-  static constexpr int NA = (227 * 1024 - RESERVED - 2 * S * B_BYTES) / A_BYTES < NA_CAP
-                                ? (227 * 1024 - RESERVED - 2 * S * B_BYTES) / A_BYTES
-                                : NA_CAP;
+  // keys and 1 KB for the barriers
+  static constexpr int NA_FIT = (227 * 1024 - 1024 - 4 * KEYS - 2 * S * B_BYTES) / A_BYTES;
+  static constexpr int NA = NA_FIT < OZ_NA_MAX ? NA_FIT : OZ_NA_MAX;
   static constexpr int CPT = BN * 4 * NGRP / EPI;                 // columns per epilogue thread
   static constexpr int TMAX = 256 / BN;                           // products per MMA (N <= 256)
   static constexpr int NBAR = 2 * NA + 4 + 2 * NBUF * S + 1;  // + the drain barrier
-  static constexpr size_t SMEM = 1024 + (size_t)NA * A_BYTES + (size_t)2 * S * B_BYTES + 8 * NBAR + 16;
+  static constexpr size_t SMEM = (size_t)NA * A_BYTES + (size_t)2 * S * B_BYTES + 8 * NBAR + 16 + 4 * KEYS;
   static_assert(NBUF * S * BN <= 512, "accumulators must fit in TMEM");
   static_assert(CPT == 8 || CPT == 16 || CPT == 32, "epilogue load width");
   static_assert(NA >= S, "a K-block of A slices must fit the ring");
@@ -579,15 +601,18 @@ struct OzCursor {
 // 7.8, 2^21 x 512 19.6 and 17.2). A Gram CTA takes 44 bytes per clock and gains
 // less (2^23 x 128: 4.66 and 4.46).
 template <int S, int MODE, int BN, int EPI, int NGRP, bool PAIR>
-__global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
+__global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
     k_ozaki_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, OzParams p) {
-  using C = OzCfg<S, BN, EPI, NGRP>;
+  using C = OzCfg<S, MODE, BN, EPI, NGRP>;
   if (p.gate && *p.gate != S) return;  // uniform for the whole grid, before any barrier or TMEM
   constexpr int NA = C::NA, NBUF = C::NBUF, CPT = C::CPT;
   constexpr int A_BYTES = C::A_BYTES, B_BYTES = C::B_BYTES;
   constexpr uint32_t ACC_COLS = S * BN;  // one accumulator buffer
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];  // 128-byte swizzle: 1024-byte atoms
+  uint8_t* smem = smem_raw;
+  // Kept as a value: with the base folded into every address as a constant the
+  // issuing thread's loop came out slower (Gram +5%).
+  asm volatile("" : "+l"(smem));
   uint8_t* sA = smem;                  // NA slots
   uint8_t* sB = sA + NA * A_BYTES;     // 2 buffers x S planes
   uint64_t* bar = (uint64_t*)(sB + 2 * S * B_BYTES);
@@ -599,7 +624,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
   uint64_t* accempty = accfull + NBUF * S;
   uint64_t* drainbar = accempty + NBUF * S;  // MMA completion on the timeout path
   uint32_t* tmem_slot = (uint32_t*)(drainbar + 1);
-  uint32_t* s_key = tmem_slot + 4;  // Q-form with p.cmax: column max keys [n]
+  uint32_t* s_key = tmem_slot + 2;  // Q-form with p.cmax: column max keys [n]
   const bool fuse_cmax = MODE == OZ_QFORM && p.cmax != nullptr;
   if (fuse_cmax)
     for (int c = threadIdx.x; c < p.n; c += blockDim.x) s_key[c] = 0u;
@@ -649,9 +674,8 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
                                          : oz_range_begin<MODE, BNU>(p, unit + 1, units);
 
   // Ring positions run on across items: A slot and its phase parity, B buffer
-  // and its parity. The single issuing threads keep their loops short (no
-  // divisions, slices and products unrolled): an MMA of N < 192 costs about
-  // as long to issue as to run.
+  // and its parity. The issuing warps keep their loops short (no divisions,
+  // slices and products unrolled).
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
@@ -723,7 +747,15 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    // The whole warp walks the loop in step and one elected lane issues: in
+    // warp-uniform code the descriptors live in the uniform registers that
+    // tcgen05.mma takes its operands from. Issued by one lane of a divergent
+    // branch, every operand was moved there first, and an MMA of N < 192 cost
+    // some 75 clocks whatever its N.
+    {
+      const bool el = elect_one();
+      const uint32_t sbase = smem_u32(smem_raw);
+      const uint32_t tmem_u = __reduce_max_sync(0xffffffffu, tmem);
       // kind::f16, BF16 A and B, FP32 accumulate, M = 128; B K-major; A K-major
       // (Gram) or MN-major (Q-form, bit 15)
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (MODE == OZ_QFORM ? 1u << 15 : 0u) |
@@ -749,22 +781,21 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
           const int ab = NGRP == 2 ? par_it : (NBUF == 2 ? (int)(gc & 1) : 0);
           const int64_t use = NGRP == 2 ? (par_it ? used1 : used0) : (NBUF == 2 ? gc >> 1 : gc);  // earlier chunks in it
           const bool wait_acc = first && use >= 1;
-          const uint32_t acc = tmem + (uint32_t)ab * ACC_COLS;
-          if (!(ok = mbar_wait(&bfull[buf], bph, p.st))) break;
-          const uint64_t db0 = sdesc(sB + buf * S * B_BYTES);
+          const uint32_t acc = tmem_u + (uint32_t)ab * ACC_COLS;
+          if (!(ok = mbar_wait_warp(&bfull[buf], bph, p.st))) break;
+          const uint64_t db0 = sdesc(sbase + (uint32_t)(NA * A_BYTES + buf * S * B_BYTES));
 #pragma unroll
           for (int s = 0; s < S; ++s) {
-            if (!(ok = mbar_wait(&afull[slot], aph, p.st))) break;
+            if (!(ok = mbar_wait_warp(&afull[slot], aph, p.st))) break;
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const uint64_t da = MODE == OZ_GRAM ? sdesc(sA + slot * A_BYTES) : sdesc_mn(sA + slot * A_BYTES);
+            const uint64_t da = MODE == OZ_GRAM ? sdesc(sbase + slot * A_BYTES) : sdesc_mn(sbase + slot * A_BYTES);
             constexpr uint64_t DA_K16 = MODE == OZ_GRAM ? 2 : 2048 >> 4;  // descriptor step per 16 k
             // Products (s, t), t = t0 .. t0+nt-1, in one MMA of N = BN nt: the
             // B slices lie back to back in shared memory (one 1024-byte pitch
             // per 8 rows throughout) and group g = s + t is the BN-column
             // accumulator at column BN g, so each product lands in its group.
             // The S - s products of slice s go in as few MMAs as N <= 256
-            // allows, split evenly: an MMA below N = 192 costs a fixed ~75
-            // clocks, so 3 + 3 beats 4 + 2 and 3 + 2 beats 4 + 1.
+            // allows, split evenly: short ones (N < 192) do not run at full rate.
             constexpr int NMMA_MAX = (S + C::TMAX - 1) / C::TMAX;
 #pragma unroll
             for (int q = 0, t0 = 0; q < NMMA_MAX && t0 < S - s; ++q) {
@@ -776,7 +807,7 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
                   // the epilogue releases each half (groups 0-3, 4..S-1) on its last group's barrier
                   const bool rep = g == 3 || g == S - 1 || g == t0 + nt - 1;
                   const int gb = g <= 3 ? 3 : S - 1;
-                  if (rep && !(ok = mbar_wait(&accempty[ab * S + gb], (uint32_t)((use - 1) & 1), p.st))) break;
+                  if (rep && !(ok = mbar_wait_warp(&accempty[ab * S + gb], (uint32_t)((use - 1) & 1), p.st))) break;
                 }
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;");
@@ -784,23 +815,27 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
               const uint32_t idesc_n = idesc | ((uint32_t)((BN * nt) >> 3) << 17);
               const uint64_t db = db0 + (uint64_t)((t0 * B_BYTES) >> 4);
               const uint32_t d = acc + (uint32_t)((s + t0) * BN);
-              mma_bf16(d, da, db, idesc_n, (s == 0 && first) ? 0u : 1u);
+              if (el) {
+                mma_bf16(d, da, db, idesc_n, (s == 0 && first) ? 0u : 1u);
 #pragma unroll
-              for (int k = 1; k < OZ_BK / 16; ++k) mma_bf16(d, da + DA_K16 * k, db + 2 * k, idesc_n, 1u);
+                for (int k = 1; k < OZ_BK / 16; ++k) mma_bf16(d, da + DA_K16 * k, db + 2 * k, idesc_n, 1u);
+              }
               t0 += nt;
             }
             if (!ok) break;
-            if (PAIR) mma_commit_pair(&aempty[slot]);
-            else mma_commit(&aempty[slot]);
-            // every product of group s is issued; the Q-form's epilogue waits on groups 3 and S-1 only
-            if (last && (MODE == OZ_GRAM || CPT != 8 || s == 3 || s == S - 1)) mma_commit(&accfull[ab * S + s]);
+            if (el) {
+              if (PAIR) mma_commit_pair(&aempty[slot]);
+              else mma_commit(&aempty[slot]);
+            }
+            // every product of group s is issued; the narrow Q-form's epilogue waits on groups 3 and S-1 only
+            if (last && (MODE == OZ_GRAM || CPT != 8 || s == 3 || s == S - 1) && el) mma_commit(&accfull[ab * S + s]);
             if (++slot == NA) {
               slot = 0;
               aph ^= 1u;
             }
           }
           if (!ok) break;
-          mma_commit(&bempty[buf]);
+          if (el) mma_commit(&bempty[buf]);
           if ((buf ^= 1) == 0) bph ^= 1u;
           if (last) {
             ++gc;
@@ -808,11 +843,12 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
           }
         }
       }
-      if (!ok) {
+      if (!ok && el) {  // the lane that issued the MMAs
         report_timeout(p.st);
         mma_commit(drainbar);  // arrives once every MMA issued so far has completed
         mbar_wait_drain(drainbar, 0);
       }
+      __syncwarp();
     }
   } else {
     const int ew = warp - 2;                            // epilogue warp
@@ -832,16 +868,15 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
       for (int c = 0; c < CPT; ++c) X[c] = Y[c] = 0;
       const int64_t row = w.i0 + q4 * 32 + lane;
       const int64_t nrow = MODE == OZ_GRAM ? p.n : p.m;
-      const int ea = 0;  // Q-form: X's column exponents live in R^-1's slices
-      // Q-form: the output columns' exponents, loaded now so that the loads
-      // overlap the drains (the Gram converts once per many chunks and keeps
-      // its registers for the accumulators)
-      constexpr int NEB = MODE == OZ_QFORM ? CPT : 1;
+      // Narrow Q-form: the output columns' exponents, loaded now so that the
+      // loads overlap the drains (the others keep their registers for the
+      // accumulators)
+      constexpr int NEB = MODE == OZ_QFORM && CPT == 8 ? CPT : 1;
       int eb[NEB];
 #pragma unroll
       for (int cc = 0; cc < NEB; ++cc) {
         const int64_t col = w.j0 + cs * CPT + cc;
-        eb[cc] = (MODE == OZ_QFORM && col < p.n) ? p.eB[col] : 0;
+        eb[cc] = (NEB > 1 && col < p.n) ? p.eB[col] : 0;
       }
       for (int c = 0; c < nchunks && ok; ++c, ++gc) {
         const int ab = NGRP == 2 ? grp : (int)(gc % NBUF);
@@ -861,29 +896,32 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
         if (MODE == OZ_QFORM && CPT == 8) {
           // two waits per chunk: groups 0-3 are complete once slice 3's
           // commit has arrived (a commit tracks every earlier MMA), the rest
-          // once the last slice's has; all loads of a half share one wait,
-          // and each half is released on its last group's barrier (fewer
-          // barrier operations per tile: the Q-form is bound by its tile
-          // pipeline's hand-offs)
+          // once the last slice's has; all loads of a half for eight columns
+          // share one wait, and each half is released on its last group's
+          // barrier once its last loads are done (fewer barrier operations per
+          // tile: the Q-form is bound by its tile pipeline's hand-offs)
 #define OZ_HALF(G0, G1)                                                      \
   if (ok) {                                                                  \
     ok = mbar_wait(&accfull[ab * S + (G1)], par, p.st);                      \
     if (ok) {                                                                \
       asm volatile("tcgen05.fence::after_thread_sync;");                     \
-      uint32_t v[4][8];                                                      \
-      _Pragma("unroll") for (int g = G0; g <= G1; ++g) tmem_ld8_nw(ta + g * BN, v[g - G0]); \
-      tmem_wait_ld();                                                        \
-      asm volatile("tcgen05.fence::before_thread_sync;");                    \
-      __syncwarp();                                                          \
-      if (lane == 0)                                                         \
-        mbar_arrive(&accempty[ab * S + (G1)]);                               \
-      if (G0 <= 0 && 0 <= G1) oz_accumulate<0, 8>(v[0 - G0], X, Y);         \
-      if (G0 <= 1 && 1 <= G1) oz_accumulate<1, 8>(v[1 - G0], X, Y);         \
-      if (G0 <= 2 && 2 <= G1) oz_accumulate<2, 8>(v[2 - G0], X, Y);         \
-      if (G0 <= 3 && 3 <= G1) oz_accumulate<3, 8>(v[3 - G0], X, Y);         \
-      if (G0 <= 4 && 4 <= G1) oz_accumulate<4, 8>(v[4 - G0 < 4 ? 4 - G0 : 0], X, Y); \
-      if (G0 <= 5 && 5 <= G1) oz_accumulate<5, 8>(v[5 - G0 < 4 ? 5 - G0 : 0], X, Y); \
-      if (G0 <= 6 && 6 <= G1) oz_accumulate<6, 8>(v[6 - G0 < 4 ? 6 - G0 : 0], X, Y); \
+      _Pragma("unroll") for (int b8 = 0; b8 < CPT; b8 += 8) {                \
+        uint32_t v[4][8];                                                    \
+        _Pragma("unroll") for (int g = G0; g <= G1; ++g) tmem_ld8_nw(ta + g * BN + b8, v[g - G0]); \
+        tmem_wait_ld();                                                      \
+        if (b8 + 8 == CPT) {                                                 \
+          asm volatile("tcgen05.fence::before_thread_sync;");                \
+          __syncwarp();                                                      \
+          if (lane == 0) mbar_arrive(&accempty[ab * S + (G1)]);              \
+        }                                                                    \
+        if (G0 <= 0 && 0 <= G1) oz_accumulate<0, 8>(v[0 - G0], X + b8, Y + b8); \
+        if (G0 <= 1 && 1 <= G1) oz_accumulate<1, 8>(v[1 - G0], X + b8, Y + b8); \
+        if (G0 <= 2 && 2 <= G1) oz_accumulate<2, 8>(v[2 - G0], X + b8, Y + b8); \
+        if (G0 <= 3 && 3 <= G1) oz_accumulate<3, 8>(v[3 - G0], X + b8, Y + b8); \
+        if (G0 <= 4 && 4 <= G1) oz_accumulate<4, 8>(v[4 - G0 < 4 ? 4 - G0 : 0], X + b8, Y + b8); \
+        if (G0 <= 5 && 5 <= G1) oz_accumulate<5, 8>(v[5 - G0 < 4 ? 5 - G0 : 0], X + b8, Y + b8); \
+        if (G0 <= 6 && 6 <= G1) oz_accumulate<6, 8>(v[6 - G0 < 4 ? 6 - G0 : 0], X + b8, Y + b8); \
+      }                                                                      \
     }                                                                        \
   }
           OZ_HALF(0, 3)
@@ -901,42 +939,65 @@ __global__ void __launch_bounds__(OzCfg<S, BN, EPI, NGRP>::THREADS, 1)
 #undef OZ_DRAIN
       }
       if (!ok) break;
-      uint32_t ck[NEB];  // Q-form: column max keys of this thread's row
+      if (MODE == OZ_GRAM) {
+        if (row < nrow) {
+          const int ea = p.eA[row];
+          double* out = p.out + (int64_t)w.split * p.n * p.n;
 #pragma unroll
-      for (int cc = 0; cc < NEB; ++cc) ck[cc] = 0u;
-      if (row < nrow) {
-        const int ea2 = MODE == OZ_GRAM ? p.eA[row] : ea;
-        double* out = MODE == OZ_GRAM ? p.out + (int64_t)w.split * p.n * p.n : p.out;
-        const int64_t ld = MODE == OZ_GRAM ? p.n : p.ldo;
-        unsigned h = 0;  // Q-form: one shift for this thread's outputs
-        if (MODE == OZ_QFORM)
-#pragma unroll
-          for (int cc = 0; cc < CPT; ++cc) h |= oz_high_bits(X[cc]);
-        const int shift = oz_group_shift(h);
-#pragma unroll
-        for (int cc = 0; cc < CPT; ++cc) {
-          const int64_t col = w.j0 + cs * CPT + cc;
-          if (col < p.n) {
-            const int e2 = MODE == OZ_QFORM ? eb[cc < NEB ? cc : 0] : p.eB[col];
-            // Gram: exact rounding; Q-form: within one ulp (far below its
-            // truncation error), with a shorter integer sequence
-            const double v = (ea2 >= EXP_NONFINITE || e2 >= EXP_NONFINITE)
-                                 ? __longlong_as_double(0x7FF8000000000000ll)
-                             : MODE == OZ_GRAM ? oz_xy_to_double(X[cc], Y[cc], ea2 + e2 - 14 - 48)
-                                               : oz_xy_to_double_group(X[cc], Y[cc], shift, ea2 + e2 - 14 - 48);
-            out[row + col * ld] = v;
-            if (MODE == OZ_QFORM && fuse_cmax) ck[cc < NEB ? cc : 0] = oz_exp_key(v);
+          for (int cc = 0; cc < CPT; ++cc) {
+            const int64_t col = w.j0 + cs * CPT + cc;
+            if (col < p.n) {
+              const int e2 = p.eB[col];
+              out[row + col * p.n] = (ea >= EXP_NONFINITE || e2 >= EXP_NONFINITE)
+                                         ? __longlong_as_double(0x7FF8000000000000ll)
+                                         : oz_xy_to_double(X[cc], Y[cc], ea + e2 - 14 - 48);
+            }
           }
         }
-      }
-      if (fuse_cmax) {
-        // the warp's 32 rows reduced per column, then one shared atomic
-        const unsigned mask = __activemask();
+      } else {
+        // A few columns at a time (four where the accumulators leave no more
+        // registers), the conversions side by side and then the rare ones again:
+        // a branch per column would serialise them.
+        constexpr int CB = CPT == 8 ? 8 : 4;
 #pragma unroll
-        for (int cc = 0; cc < NEB; ++cc) {
-          const uint32_t mk = __reduce_max_sync(mask, ck[cc]);
-          const int64_t col = w.j0 + cs * CPT + cc;
-          if (lane == __ffs(mask) - 1 && col < p.n && mk != 0u) atomicMax(&s_key[col], mk);
+        for (int cb = 0; cb < CPT; cb += CB) {
+          unsigned h = 0;  // one shift for these outputs of the thread
+#pragma unroll
+          for (int cc = cb; cc < cb + CB; ++cc) h |= oz_high_bits(X[cc]);
+          const int shift = oz_group_shift(h);
+          const int64_t col0 = w.j0 + cs * CPT + cb;
+          const int ncol = (int)min((int64_t)CB, p.n - col0);  // may be negative
+          double v[CB];
+          unsigned rare = 0;
+#pragma unroll
+          for (int cc = 0; cc < CB; ++cc) {
+            const int e2 = NEB > 1 ? eb[cb + cc < NEB ? cb + cc : 0] : (cc < ncol ? p.eB[col0 + cc] : 0);
+            bool fine;
+            v[cc] = oz_xy_to_double_group_fast(X[cb + cc], Y[cb + cc], shift, e2 - 14 - 48, &fine);
+            if (!fine && cc < ncol) rare |= 1u << cc;
+          }
+          if (rare != 0) {
+#pragma unroll
+            for (int cc = 0; cc < CB; ++cc)
+              if (rare >> cc & 1) {
+                const int e2 = p.eB[col0 + cc];
+                v[cc] = e2 >= EXP_NONFINITE ? __longlong_as_double(0x7FF8000000000000ll)
+                                            : oz_xy_to_double_group(X[cb + cc], Y[cb + cc], shift, e2 - 14 - 48);
+              }
+          }
+          if (row < nrow) {
+            double* out = p.out + row + col0 * p.ldo;
+#pragma unroll
+            for (int cc = 0; cc < CB; ++cc)
+              if (cc < ncol) out[cc * p.ldo] = v[cc];
+          }
+          if (fuse_cmax) {  // the warp's 32 rows reduced per column, then one shared atomic
+#pragma unroll
+            for (int cc = 0; cc < CB; ++cc) {
+              const uint32_t mk = __reduce_max_sync(0xffffffffu, row < nrow ? oz_exp_key(v[cc]) : 0u);
+              if (lane == 0 && cc < ncol && mk != 0u) atomicMax(&s_key[col0 + cc], mk);
+            }
+          }
         }
       }
     }
@@ -1042,9 +1103,9 @@ EncodeTiledFn encode_fn() {
 
 template <int S, int MODE, int BN, int EPI, int NGRP, bool PAIR>
 cudaError_t launch_oz(const CUtensorMap& a, const CUtensorMap& b, const OzParams& p, int64_t sms, cudaStream_t s) {
-  using Cfg = OzCfg<S, BN, EPI, NGRP>;
-  // the Q-form also holds the column max keys (after the TMEM slot)
-  constexpr size_t SMEM = Cfg::SMEM + (MODE == OZ_QFORM ? 4 * OZ_CMAX_N + 16 : 0);
+  using Cfg = OzCfg<S, MODE, BN, EPI, NGRP>;
+  constexpr size_t SMEM = Cfg::SMEM;
+  static_assert(MODE != OZ_QFORM || Cfg::KEYS >= OZ_CMAX_N, "column max keys");
   static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
   auto kern = k_ozaki_gemm<S, MODE, BN, EPI, NGRP, PAIR>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
@@ -1101,11 +1162,25 @@ bool oz_gram_pairs(int n) {
   const int nj = (int)ceil_div(n, OZ_GRAM_BN), np = (int)ceil_div(n, 2 * OZ_GRAM_BN);
   return 2.0 * oz_gram_tiles(np, 1) <= 1.15 * oz_gram_tiles(nj, OZ_BM / OZ_GRAM_BN);
 }
-bool oz_qform_pairs(int n) {
-  double paired = 0.0, single = 0.0;  // costs in the ranges' model, K-blocks plus one per tile
-  for (int j = 0; j < n; j += OZ_QFORM_BN) single += ceil_div(j + OZ_QFORM_BN, OZ_BK) + 1;
-  for (int j = 0; j < n; j += 2 * OZ_QFORM_BN) paired += 2.0 * (ceil_div(j + 2 * OZ_QFORM_BN, OZ_BK) + 1);
-  return paired <= 1.15 * single;
+
+// The Q-form's shape: 32-column tiles on single CTAs or on pairs, or 64-column
+// tiles on pairs. A wider tile reuses each A slice more often: per K-block the
+// shared-memory port (128 bytes per clock) serves the MMAs' operands and the
+// incoming slices in 2850 clocks for 32 columns and 4300 for 64; but its
+// accumulators fill TMEM (one buffer), and a ragged last tile costs more. Costs
+// per row tile, in K-blocks plus half a one per tile, of a pair's narrow tiles;
+// singles 1.2 times (their A traffic), wide ones 1.65 times. Measured at 2^27
+// entries, us for both Q-forms, narrow pairs and wide: n = 128 1334, 1406; 200
+// 2463, 2392; 256 1945, 1904; 320 2292, 2723; 512 3281, 2981; 768 4609, 3990.
+enum OzQShape { OZ_Q_SINGLE, OZ_Q_PAIR, OZ_Q_WIDE };
+OzQShape oz_qform_shape(int n) {
+  auto cost = [n](int bn) {
+    double c = 0.0;
+    for (int j = 0; j < n; j += bn) c += std::min(ceil_div(j + bn, OZ_BK), ceil_div(n, OZ_BK)) + 0.5;
+    return c;
+  };
+  const double single = 0.6 * cost(OZ_QFORM_BN), pair = cost(2 * OZ_QFORM_BN), wide = 1.65 * cost(2 * OZ_QFORM_BN_WIDE);
+  return wide < pair && wide < single ? OZ_Q_WIDE : (pair <= single ? OZ_Q_PAIR : OZ_Q_SINGLE);
 }
 
 // Row ranges of the Gram: its items (ranges x tiles) all cost the same and are
@@ -1182,7 +1257,8 @@ cudaError_t ozaki_make_maps(OzMaps& maps, int64_t m, int n, int S, void* planes,
   static_assert(sizeof(CUtensorMap) <= sizeof(OzMaps::col_a), "tensor map storage");
   bool ok = make_tiled((CUtensorMap*)maps.col_a, OZ_BM) && make_tiled((CUtensorMap*)maps.col_b, OZ_GRAM_BN) &&
             make_tiled((CUtensorMap*)maps.col_a_mn, OZ_BK) &&
-            make((CUtensorMap*)maps.rinv_b, rinv_planes, (uint64_t)g.np, (uint64_t)n, OZ_QFORM_BN);
+            make((CUtensorMap*)maps.rinv_b, rinv_planes, (uint64_t)g.np, (uint64_t)n, OZ_QFORM_BN) &&
+            make((CUtensorMap*)maps.rinv_b_wide, rinv_planes, (uint64_t)g.np, (uint64_t)n, OZ_QFORM_BN_WIDE);
   return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -1271,19 +1347,25 @@ cudaError_t ozaki_qform(const OzMaps& maps, int64_t m, int n, int S, const int* 
   p.out = Q;
   p.ldo = ldq;
   p.st = st;
-  const bool pair = oz_qform_pairs(n);
-  p.ntile_j = (int)ceil_div(n, pair ? 2 * OZ_QFORM_BN : OZ_QFORM_BN);
+  const OzQShape shape = oz_qform_shape(n);
+  const bool wide = shape == OZ_Q_WIDE, pair = shape != OZ_Q_SINGLE;
+  const int bn = wide ? OZ_QFORM_BN_WIDE : OZ_QFORM_BN;
+  p.ntile_j = (int)ceil_div(n, pair ? 2 * bn : bn);
   p.ntiles = 1;
   p.nitems = (int64_t)p.ntile_j * ceil_div(m, OZ_BM);
   p.gate = gate;
   const CUtensorMap& a = *(const CUtensorMap*)maps.col_a_mn;
-  const CUtensorMap& b = *(const CUtensorMap*)maps.rinv_b;
+  const CUtensorMap& b = *(const CUtensorMap*)(wide ? maps.rinv_b_wide : maps.rinv_b);
   const int64_t sms = sm_count_oz();
-  constexpr int BN = OZ_QFORM_BN, EPI = OZ_QFORM_EPI, GRP = OZ_QFORM_GRP;
-  return pair ? (S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s)
-                        : launch_oz<6, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s))
-              : (S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s)
-                        : launch_oz<6, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s));
+  constexpr int BN = OZ_QFORM_BN, BNW = OZ_QFORM_BN_WIDE, EPI = OZ_QFORM_EPI, GRP = OZ_QFORM_GRP;
+  if (wide)
+    return S == 7 ? launch_oz<7, OZ_QFORM, BNW, EPI, GRP, true>(a, b, p, sms, s)
+                  : launch_oz<6, OZ_QFORM, BNW, EPI, GRP, true>(a, b, p, sms, s);
+  if (pair)
+    return S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s)
+                  : launch_oz<6, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s);
+  return S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s)
+                : launch_oz<6, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s);
 }
 
 cudaError_t ozaki_route(const int* cexp, const double* W, int64_t ldw, int n, int64_t m, int* gate, bool keep,
