@@ -129,8 +129,8 @@ __device__ __forceinline__ void bar_wait(int id) {
 
 // The diagonal tile's factorization with divisions, for pivots outside the
 // reciprocal's range and for breakdowns (reported, and spread as NaN).
-__device__ __noinline__ void factor_tile_div(double* t, Pair e, double* Vd, double* Ld, double* Z, double* dd, int lane,
-                                             int nlive, DevStatus* st, int pass, long long off) {
+__device__ __noinline__ void factor_tile_div(double* t, Pair e, double* Ld, double* Z, double* dd, int lane, int nlive,
+                                             DevStatus* st, int pass, long long off) {
   const int r = lane & 7, g = lane >> 3, c0 = 2 * g, c1 = 2 * g + 1;
   __syncwarp();
   tile_put(t, r, g, e);
@@ -147,7 +147,6 @@ __device__ __noinline__ void factor_tile_div(double* t, Pair e, double* Vd, doub
     }
     if (lane == 0) dd[k] = d;
     const double w = ar / d;
-    if (c0 == k || c1 == k) Vd[r * TLD + k] = r < k ? 0.0 : (r == k ? d : ar);
     if (c0 == k) l.x = w;
     if (c1 == k) l.y = w;
     __syncwarp();
@@ -163,42 +162,30 @@ __device__ __noinline__ void factor_tile_div(double* t, Pair e, double* Vd, doub
 }
 
 // Factors the diagonal tile (this lane's elements e, t its shared memory): Z,
-// Lu, V and D of the block (dd: D, then its reciprocals). Warp 0. Each lane
-// forms the pivot's reciprocal itself. A step's chain is one FMA (the element
-// of column k + 1 first), its exchange through shared memory, the reciprocal
-// in integers and the product; the other element's FMA runs beside the next
-// reciprocal, and nothing on the chain branches: the pivots' range is looked
-// at once, at the end. V's column k and 1/d are published step by step for
-// the panel warps.
-__device__ __forceinline__ void factor_tile(double* t, Pair e, double* Vd, double* Ld, double* Z, double* dd,
-                                            int* exact, int lane, int nlive, DevStatus* st, int pass, long long off) {
+// Lu and D of the block (dd: D, then its reciprocals). Warp 0. Each lane forms
+// the pivot's reciprocal itself. A step's chain is one FMA (the element of
+// column k + 1 first), its exchange through shared memory, the reciprocal in
+// integers and the product; the other element's FMA runs beside the next
+// reciprocal, and nothing on the chain branches: the pivots' range is looked at
+// once, at the end. Lu's columns are published step by step for the panel warps.
+__device__ __forceinline__ void factor_tile(double* t, Pair e, double* Ld, double* Z, double* dd, int* exact, int lane,
+                                            int nlive, DevStatus* st, int pass, long long off) {
   const int r = lane & 7, g = lane >> 3, c0 = 2 * g, c1 = 2 * g + 1;
   const Pair e0 = e;
-  Pair l{0.0, 0.0};
   bool ok = true;
   tile_put(t, r, g, e);
+  tile_put(Ld, r, g, {c0 == r ? 1.0 : 0.0, c1 == r ? 1.0 : 0.0});
   __syncwarp();
   double d = t[0];
 #pragma unroll
   for (int k = 0; k < TB; ++k) {
-    if (c0 == k || c1 == k) Vd[r * TLD + k] = r < k ? 0.0 : (c0 == k ? e.x : e.y);
     const double y = pivot_rcp(d);
     ok = ok && pivot_rcp_ok(d);
     __syncwarp();  // step k - 1's elements are all in place
     const double ar = t[r * TLD + k];
     const double b0 = t[(c0 > k ? c0 : k) * TLD + (c0 > k ? k : c0)];
     const double b1 = t[(c1 > k ? c1 : k) * TLD + (c1 > k ? k : c1)];
-    const double w = ar * y;
-    if (lane == 0) {
-      dd[k] = d;
-      dd[TB + k] = y;
-      if (k == TB - 1) *exact = !ok;
-    }
-    if (c0 == k) l.x = w;
-    if (c1 == k) l.y = w;
-    __syncwarp();  // the step's reads are done, and column k is published
-    bar_arrive(PANEL_BAR + k);
-    if (k == TB - 1) break;
+    const double w = ar * y;  // Lu's column k
     const bool below = r > k;
     const double s0 = c0 == k ? 1.0 : b0, s1 = c1 == k ? 1.0 : b1;
     const double f0 = c0 == k ? 0.0 : e.x, f1 = c1 == k ? 0.0 : e.y;
@@ -211,22 +198,34 @@ __device__ __forceinline__ void factor_tile(double* t, Pair e, double* Vd, doubl
       const double v = fma(nw, s1, f1);
       if (below) t[r * TLD + c1] = e.y = v;
     };
-    if ((k + 1) & 1) second();
-    else first();
+    __syncwarp();  // the step's reads are done
+    if (k < TB - 1) {
+      if ((k + 1) & 1) second();
+      else first();
+      __syncwarp();
+    }
+    const double dk = d;
+    if (k < TB - 1) {
+      d = t[(k + 1) * TLD + k + 1];
+      if ((k + 1) & 1) first();
+      else second();
+    }
+    if (below && (c0 == k || c1 == k)) Ld[r * TLD + k] = w;
+    if (lane == 0) {
+      dd[k] = dk;
+      dd[TB + k] = y;
+      if (k == TB - 1) *exact = !ok;
+    }
     __syncwarp();
-    d = t[(k + 1) * TLD + k + 1];
-    if ((k + 1) & 1) first();
-    else second();
+    bar_arrive(PANEL_BAR + k);
   }
   if (!ok) {
-    factor_tile_div(t, e0, Vd, Ld, Z, dd, lane, nlive, st, pass, off);
+    factor_tile_div(t, e0, Ld, Z, dd, lane, nlive, st, pass, off);
     __syncwarp();
     bar_wait(PANEL_BAR + TB);
     return;
   }
-  // unit lower
-  tile_put(Z, r, g, {c0 < r ? e.x : (c0 == r ? 1.0 : 0.0), c1 < r ? e.y : (c1 == r ? 1.0 : 0.0)});
-  tile_put(Ld, r, g, {c0 < r ? l.x : (c0 == r ? 1.0 : 0.0), c1 < r ? l.y : (c1 == r ? 1.0 : 0.0)});
+  tile_put(Z, r, g, {c0 < r ? e.x : (c0 == r ? 1.0 : 0.0), c1 < r ? e.y : (c1 == r ? 1.0 : 0.0)});  // unit lower
 }
 
 __global__ void __launch_bounds__(LT, 1)
@@ -283,7 +282,6 @@ __global__ void __launch_bounds__(LT, 1)
   // and their way to the cluster. Run by the owner's whole CTA.
   auto lead_column = [&](int p) {
     double* tb = tile_base(p / C);
-    double* Vd = slot_tile(sm.V, p, p);
     double* Ld = slot_tile(sm.Lu, p, p);
     double* dd = sm.dg + (p % SLOTS) * 2 * TB;
     double* Z = sm.Z + (p & 1) * TSZ;
@@ -299,7 +297,7 @@ __global__ void __launch_bounds__(LT, 1)
         e.x += h.x + h1.x;
         e.y += h.y + h1.y;
       }
-      factor_tile(tb, e, Vd, Ld, Z, dd, &s_exact, lane, n - p * TB, st, pass, off + (long long)p * TB);
+      factor_tile(tb, e, Ld, Z, dd, &s_exact, lane, n - p * TB, st, pass, off + (long long)p * TB);
       __syncwarp();
       const Pair ld = tile_get(Ld, r, g);
       const double dl = dd[lane & (TB - 1)];
@@ -329,20 +327,22 @@ __global__ void __launch_bounds__(LT, 1)
           if (p) tile_sub(v[u], slot_tile(sm.Lu, p - 1, i), Vn, r, g);
           tile_put(tl, r, g, v[u]);  // for a second solve with divisions
         }
-        // column k of V is final once the columns before it are subtracted
+        // V(r, c) -= V(r, k) Lu(c, k): column k is final once the columns before it are subtracted
 #pragma unroll
         for (int k = 0; k < TB; ++k) {
           bar_wait(PANEL_BAR + k);
-          const double y = dd[TB + k], b0 = Vd[2 * g * TLD + k], b1 = Vd[(2 * g + 1) * TLD + k];
+          if (k == TB - 1) break;
+          const double b0 = Ld[2 * g * TLD + k], b1 = Ld[(2 * g + 1) * TLD + k];
 #pragma unroll
           for (int u = 0; u < U; ++u) {
-            const double w = __shfl_sync(0xffffffffu, (k & 1) ? v[u].y : v[u].x, r + 8 * (k >> 1)) * y;
-            if (2 * g == k) l[u].x = w;
-            if (2 * g + 1 == k) l[u].y = w;
-            if (k < 6) v[u].x = 2 * g > k ? fma(-w, b0, v[u].x) : v[u].x;
-            if (k < 7) v[u].y = 2 * g + 1 > k ? fma(-w, b1, v[u].y) : v[u].y;
+            const double vk = __shfl_sync(0xffffffffu, (k & 1) ? v[u].y : v[u].x, r + 8 * (k >> 1));
+            if (k < 6) v[u].x = 2 * g > k ? fma(-vk, b0, v[u].x) : v[u].x;
+            v[u].y = 2 * g + 1 > k ? fma(-vk, b1, v[u].y) : v[u].y;
           }
         }
+        const Pair y = *reinterpret_cast<const double2*>(dd + TB + 2 * g);
+#pragma unroll
+        for (int u = 0; u < U; ++u) l[u] = {v[u].x * y.x, v[u].y * y.y};
       };
       if (nt == 0) {
         for (int k = 0; k < TB; ++k) bar_wait(PANEL_BAR + k);
@@ -363,13 +363,12 @@ __global__ void __launch_bounds__(LT, 1)
         if (again) {
           v[u] = tile_get(tb + (i - p) * TSZ, r, g);
 #pragma unroll
-          for (int k = 0; k < TB; ++k) {
-            const double w = __shfl_sync(0xffffffffu, (k & 1) ? v[u].y : v[u].x, r + 8 * (k >> 1)) / dd[k];
-            if (2 * g == k) l[u].x = w;
-            if (2 * g + 1 == k) l[u].y = w;
-            if (2 * g > k) v[u].x = fma(-w, Vd[2 * g * TLD + k], v[u].x);
-            if (2 * g + 1 > k) v[u].y = fma(-w, Vd[(2 * g + 1) * TLD + k], v[u].y);
+          for (int k = 0; k < TB - 1; ++k) {
+            const double vk = __shfl_sync(0xffffffffu, (k & 1) ? v[u].y : v[u].x, r + 8 * (k >> 1));
+            if (2 * g > k) v[u].x = fma(-vk, Ld[2 * g * TLD + k], v[u].x);
+            if (2 * g + 1 > k) v[u].y = fma(-vk, Ld[(2 * g + 1) * TLD + k], v[u].y);
           }
+          l[u] = {v[u].x / dd[2 * g], v[u].y / dd[2 * g + 1]};
         }
         double* Vi = slot_tile(sm.V, p, i);
         double* Li = slot_tile(sm.Lu, p, i);
