@@ -23,14 +23,15 @@
 // brings that column up to date; one warp factors its diagonal tile while six
 // others follow it column by column with V and Lu of the tiles below, and send
 // Lu to every CTA of the cluster and V(j) to the owner of column j (distributed
-// shared memory). Only then does it join the others in the rest of step p. One split cluster barrier per step: a CTA
-// arrives when it has entered the step (the owner, when its panel is sent)
-// and waits when it has finished it, so panels live in three slots (a panel is
-// overwritten two steps after every CTA has arrived past its last use).
+// shared memory). Only then does it join the others in the rest of step p. One
+// split cluster barrier per step: a CTA arrives when it has entered the step
+// (the owner, when its panel is sent) and waits when it has finished it, so
+// panels live in three slots (a panel is overwritten two steps after every CTA
+// has arrived past its last use).
 //
 // Measured, us per CholInv back to back (before: one CTA per 64 columns with a
 // rank-1 step and a block barrier per column, GEMM launches above that):
-// n = 16: 25 -> 13, 32: 41 -> 20, 64: 64 -> 38, 100: 222 -> 70, 128: 238 -> 102.
+// n = 16: 22 -> 13, 32: 37 -> 21, 64: 64 -> 39, 100: 222 -> 72, 128: 238 -> 99.
 #include <algorithm>
 #include <type_traits>
 
@@ -118,7 +119,8 @@ struct LeafSmem {
 // divisions. Warp 0 factors and PW = 6 warps solve panel tiles; warp 4, on
 // warp 0's SM partition, stays out. (With three panel warps the factorization
 // runs undisturbed, 4000 clocks against up to 5000, but the panel then takes
-// longer than it: 45 against 41 us at n = 64, 126 against 102 us at n = 128.)
+// longer than it: 45 against 41 us at n = 64, 126 against 102 us at n = 128,
+// with 21 FP64 instructions to a panel tile; it has 15 now.)
 constexpr int PW = 6, PANEL_BAR = 2, PANEL_THREADS = 32 * (1 + PW);
 __device__ __forceinline__ void bar_arrive(int id) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(PANEL_THREADS) : "memory");
