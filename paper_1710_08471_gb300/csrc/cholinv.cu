@@ -18,8 +18,9 @@ namespace {
 
 constexpr int NB = CHOLINV_BASE;
 
-__global__ void k_transpose_lower(const double* __restrict__ L, int64_t ldl, int n, double* __restrict__ R,
+__global__ void k_transpose_lower(const double* L, int64_t ldl, int n, double* R,
                                   int64_t ldr) {
+  grid_chain();
   __shared__ double tile[32][33];
   const int bi = blockIdx.x * 32, bj = blockIdx.y * 32;  // R block (rows bi.., cols bj..)
   // read L block (rows bj.., cols bi..) coalesced along its rows
@@ -34,7 +35,8 @@ __global__ void k_transpose_lower(const double* __restrict__ L, int64_t ldl, int
   }
 }
 
-__global__ void k_copy_upper(const double* __restrict__ X, int64_t ldx, int n, double* __restrict__ R, int64_t ldr) {
+__global__ void k_copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr) {
+  grid_chain();
   const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i < n) R[i + (int64_t)j * ldr] = (i <= j) ? X[i + (int64_t)j * ldx] : 0.0;
 }
@@ -198,14 +200,16 @@ cudaError_t add_shift(double* W, int64_t ldw, int n, int64_t m, cudaStream_t s) 
 
 cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int64_t ldr, cudaStream_t s) {
   dim3 grid((unsigned)ceil_div(n, 32), (unsigned)ceil_div(n, 32));
-  k_transpose_lower<<<grid, dim3(32, 8), 0, s>>>(L, ldl, n, R, ldr);
+  cudaError_t e = launch_chained(k_transpose_lower, grid, dim3(32, 8), 0, s, dim3(1), true, L, ldl, n, R, ldr);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr, cudaStream_t s) {
   dim3 grid((unsigned)ceil_div(n, 128), (unsigned)n);
-  k_copy_upper<<<grid, 128, 0, s>>>(X, ldx, n, R, ldr);
+  cudaError_t e = launch_chained(k_copy_upper, grid, dim3(128), 0, s, dim3(1), true, X, ldx, n, R, ldr);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }

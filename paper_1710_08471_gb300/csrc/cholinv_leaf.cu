@@ -233,6 +233,7 @@ __device__ __forceinline__ void factor_tile(double* t, Pair e, double* Ld, doubl
 __global__ void __launch_bounds__(LT, 1)
     k_cholinv_leaf(const double* W, int64_t ldw, int n, double* L, int64_t ldl, double* Y, int64_t ldy, double* Rt,
                    int64_t ldrt, double* Rp, int rpw, DevStatus* st, int pass, long long off) {
+  grid_chain();
   extern __shared__ __align__(16) double smem[];
   __shared__ int s_exact;  // a pivot of the panel factored last needs real divisions
   const int C = (int)cluster_size(), me = (int)cluster_rank();
@@ -546,18 +547,8 @@ cudaError_t cholinv_leaf(int n, const double* W, int64_t ldw, double* L, int64_t
   if (sm > LEAF_SMEM_MAX) return cudaErrorInvalidValue;
   cudaError_t e = cudaFuncSetAttribute(k_cholinv_leaf, cudaFuncAttributeMaxDynamicSharedMemorySize, LEAF_SMEM_MAX);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)C);
-  cfg.blockDim = dim3(LT);
-  cfg.dynamicSmemBytes = sm;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = (unsigned)C;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_cholinv_leaf, W, ldw, n, L, ldl, Y, ldy, Rt, ldrt, Rp, rpw, st, pass, off);
+  e = launch_chained(k_cholinv_leaf, dim3((unsigned)C), dim3(LT), sm, s, dim3((unsigned)C), true, W, ldw, n, L, ldl, Y,
+                     ldy, Rt, ldrt, Rp, rpw, st, pass, off);
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();

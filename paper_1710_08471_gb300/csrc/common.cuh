@@ -39,6 +39,56 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
+// The kernels of a factorization follow one another on one stream, and the
+// small ones take a few microseconds each, about as long as the stream needs
+// to drain one grid and start the next. They are launched with launch_chained,
+// which lets a grid be set up on the SMs while its predecessor still runs, and
+// open with grid_chain(): wait until the predecessor has completed and its
+// writes are visible, then let the successor be set up. Since no grid ends
+// before its own wait, completion stays in stream order, also for what is read
+// and overwritten. Pointers of these kernels carry no __restrict__: a load
+// through the read-only path could be moved above the wait. (us per pass, whole
+// factorizations: least squares of 1024 x 16 79 -> 61, 4096 x 64 202 -> 192,
+// least squares of 131601 x 256 in split precision 2035 -> 2006.)
+__device__ __forceinline__ void grid_chain() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Whether a grid of that many CTAs is set up early. One that fills the SMs is
+// not: while its predecessor holds some of them, its CTAs pile up on the rest.
+// (777 columns in FP64: 15.4 ms, with every GEMM set up early 16.1. The Gram and
+// the Q-form pass twice their CTAs: these run for long on an SM each, and at
+// 4096 x 64 early ones cost 10 us. The 128 x 128 GEMMs of CholInv gain at up to
+// an SM each, 12 us of 2017 at 131601 x 256.)
+inline bool chain_early(int64_t ctas) {
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return ctas <= sms;
+}
+
+// Launches kern (as a cluster where that has more than one CTA).
+template <typename... P, typename... Args>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, dim3 cluster, bool early,
+                           Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2]{};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cluster.x;
+  at[1].val.clusterDim.y = cluster.y;
+  at[1].val.clusterDim.z = cluster.z;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster.x * cluster.y * cluster.z > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 }  // namespace cqr2

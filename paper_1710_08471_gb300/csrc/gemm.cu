@@ -45,9 +45,10 @@ __device__ __forceinline__ double ld_remote(const double* p, uint32_t rank) {
 
 template <int T, bool TA, bool TB>
 __global__ void __launch_bounds__(4 * T) k_gemm_f64(int64_t M, int64_t N, int64_t K, double alpha,
-                                                    const double* __restrict__ A, int64_t lda,
-                                                    const double* __restrict__ B, int64_t ldb, double beta,
-                                                    double* __restrict__ C, int64_t ldc, unsigned flags, int ksplit) {
+                                                    const double* A, int64_t lda,
+                                                    const double* B, int64_t ldb, double beta,
+                                                    double* C, int64_t ldc, unsigned flags, int ksplit) {
+  grid_chain();
   constexpr int NT = 4 * T, TX = T / 4, NC = T / 16, PITCH = T + 1, NQ = 4;
   static_assert(T * BK / NT == NQ, "elements per thread of a staged slice");
   __shared__ double smem[4 * BK * PITCH];
@@ -220,17 +221,10 @@ __global__ void __launch_bounds__(4 * T) k_gemm_f64(int64_t M, int64_t N, int64_
 template <int T, bool TA, bool TB>
 cudaError_t launch_gemm(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
                         int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, int ks, cudaStream_t s) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)ceil_div(M, T), (unsigned)ceil_div(N, T), (unsigned)ks);
-  cfg.blockDim = dim3(4 * T);
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = at.val.clusterDim.y = 1;
-  at.val.clusterDim.z = (unsigned)ks;
-  cfg.attrs = &at;
-  cfg.numAttrs = ks > 1 ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_gemm_f64<T, TA, TB>, M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, ks);
+  const dim3 grid((unsigned)ceil_div(M, T), (unsigned)ceil_div(N, T), (unsigned)ks);
+  cudaError_t e = launch_chained(k_gemm_f64<T, TA, TB>, grid, dim3(4 * T), 0, s, dim3(1, 1, (unsigned)ks),
+                                 chain_early((int64_t)grid.x * grid.y * grid.z), M, N, K, alpha, A, lda, B, ldb, beta, C,
+                                 ldc, flags, ks);
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
@@ -300,8 +294,9 @@ cudaError_t gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const double
 // needs a split-k launch and its reduction for this 2 n^3 / 6 flop product.
 constexpr int TRMM_PARTS = 4;
 __global__ void __launch_bounds__(TRMM_PARTS * TRMM_SMALL_MAX)
-    k_trmm_upper_small(int n, const double* __restrict__ A, int64_t lda, bool a_trans, const double* __restrict__ B,
-                       int64_t ldb, double* __restrict__ C, int64_t ldc) {
+    k_trmm_upper_small(int n, const double* A, int64_t lda, bool a_trans, const double* B,
+                       int64_t ldb, double* C, int64_t ldc) {
+  grid_chain();
   __shared__ double bj[TRMM_SMALL_MAX];
   const int j = blockIdx.x, t = threadIdx.x, i = t / TRMM_PARTS, q = t % TRMM_PARTS;
   for (int k = t; k <= j; k += blockDim.x) bj[k] = B[k + (int64_t)j * ldb];
@@ -327,7 +322,9 @@ cudaError_t trmm_upper_small(int n, const double* A, int64_t lda, bool a_trans, 
                              double* C, int64_t ldc, cudaStream_t s) {
   if (n < 1 || n > TRMM_SMALL_MAX) return cudaErrorInvalidValue;
   const int threads = (TRMM_PARTS * n + 31) / 32 * 32;
-  k_trmm_upper_small<<<n, threads, 0, s>>>(n, A, lda, a_trans, B, ldb, C, ldc);
+  cudaError_t e = launch_chained(k_trmm_upper_small, dim3((unsigned)n), dim3((unsigned)threads), 0, s, dim3(1), true,
+                                 n, A, lda, a_trans, B, ldb, C, ldc);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }

@@ -129,8 +129,9 @@ __device__ __forceinline__ void off_item(const double* __restrict__ A, int64_t l
 // One diagonal tile (n <= 128) of at most MAXS slots per thread.
 template <int MAXS>
 __global__ void __launch_bounds__(NT, MAXS <= 8 ? 3 : (MAXS <= 16 ? 2 : 1))
-    k_gram_diag(const double* __restrict__ A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T,
-                double* __restrict__ partial) {
+    k_gram_diag(const double* A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T,
+                double* partial) {
+  grid_chain();
   extern __shared__ double smem[];
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_split, r1 = min(m, r0 + rows_per_split);
   diag_item<MAXS>(A, lda, r0, r1, 0, n, smem, partial + (int64_t)blockIdx.x * T * T, T);
@@ -182,9 +183,10 @@ __global__ void __launch_bounds__(NT, 1)
 // instruction in full, so one thread per element and hundreds of ranges left
 // most of the GPU idle).
 constexpr int GRAM_RC = 8;
-__global__ void __launch_bounds__(32 * GRAM_RC) k_gram_reduce(const double* __restrict__ partial, int64_t nsplit,
+__global__ void __launch_bounds__(32 * GRAM_RC) k_gram_reduce(const double* partial, int64_t nsplit,
                                                               int T, int ntile, int ntiles_total, int n,
-                                                              double* __restrict__ W, int64_t ldw) {
+                                                              double* W, int64_t ldw) {
+  grid_chain();
   __shared__ double part[GRAM_RC][32];
   const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
   const int i = blockIdx.x * 32 + lane;
@@ -226,7 +228,9 @@ cudaError_t launch_diag(const double* A, int64_t lda, int64_t m, int n, const Gr
   cudaError_t e = cudaFuncSetAttribute(k_gram_diag<MAXS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(2 * KC * 129 * sizeof(double)));
   if (e != cudaSuccess) return e;
-  k_gram_diag<MAXS><<<(unsigned)g.nsplit, NT, sm, s>>>(A, lda, m, n, g.rows_per_split, g.T, partial);
+  e = launch_chained(k_gram_diag<MAXS>, dim3((unsigned)g.nsplit), dim3(NT), sm, s, dim3(1),
+                     chain_early(2 * g.nsplit), A, lda, m, n, g.rows_per_split, g.T, partial);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
@@ -285,7 +289,9 @@ cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const 
 cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw, cudaStream_t s) {
   dim3 block(32 * GRAM_RC);
   dim3 grid((unsigned)ceil_div(n, 32), (unsigned)n);
-  k_gram_reduce<<<grid, block, 0, s>>>(partial, g.nsplit, g.T, g.ntile, g.ntiles_total, n, W, ldw);
+  cudaError_t e = launch_chained(k_gram_reduce, grid, block, 0, s, dim3(1), true, partial, g.nsplit, g.T, g.ntile,
+                                 g.ntiles_total, n, W, ldw);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }

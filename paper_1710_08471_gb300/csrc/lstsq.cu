@@ -23,9 +23,10 @@ namespace {
 // 131601 x 256: 280 -> 69 us (83% of the FP64 pipe); 50021 x 100: 86 -> 15 us.
 constexpr int GT = 256, GW = GT / 32, GC = 8;
 
-__global__ void __launch_bounds__(GT) k_gemv_t_partial(const double* __restrict__ Q, int64_t ldq, int64_t m, int n,
-                                                       const double* __restrict__ b, int64_t rows_per, int gpc,
-                                                       double* __restrict__ partial) {
+__global__ void __launch_bounds__(GT) k_gemv_t_partial(const double* Q, int64_t ldq, int64_t m, int n,
+                                                       const double* b, int64_t rows_per, int gpc,
+                                                       double* partial) {
+  grid_chain();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t split = (int64_t)blockIdx.x * (GW / gpc) + warp / gpc;
   const int c0 = ((int)blockIdx.y * gpc + warp % gpc) * GC;
@@ -97,9 +98,10 @@ __host__ __device__ constexpr int solve_width(int n) {
   return w;
 }
 
-__global__ void __launch_bounds__(ST) k_lstsq_solve(const double* __restrict__ partial, int64_t nsplit, int n,
-                                                    const double* __restrict__ R, int64_t ldr,
-                                                    double* __restrict__ x) {
+__global__ void __launch_bounds__(ST) k_lstsq_solve(const double* partial, int64_t nsplit, int n,
+                                                    const double* R, int64_t ldr,
+                                                    double* x) {
+  grid_chain();
   extern __shared__ double c[];  // c[n], then ST partial sums where columns' sums are shared
   double* ps = c + n;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -227,7 +229,9 @@ cudaError_t gemv_t_partials(const double* Q, int64_t ldq, int64_t m, int n, cons
   const int gpc = gemv_groups(n);
   const int64_t rows_per = ceil_div(ceil_div(m, nsplit), 32) * 32;  // ranges start on 256-byte lines
   dim3 grid((unsigned)(nsplit / (GW / gpc)), (unsigned)ceil_div(n, gpc * GC));
-  k_gemv_t_partial<<<grid, GT, 0, s>>>(Q, ldq, m, n, b, rows_per, gpc, partial);
+  cudaError_t e = launch_chained(k_gemv_t_partial, grid, dim3(GT), 0, s, dim3(1),
+                                 chain_early((int64_t)grid.x * grid.y), Q, ldq, m, n, b, rows_per, gpc, partial);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
@@ -239,7 +243,9 @@ cudaError_t lstsq_solve(const double* partial, int64_t nsplit, int n, const doub
     cudaError_t e = cudaFuncSetAttribute(k_lstsq_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
-  k_lstsq_solve<<<1, ST, sm, s>>>(partial, nsplit, n, R, ldr, x);
+  cudaError_t e = launch_chained(k_lstsq_solve, dim3(1), dim3(ST), sm, s, dim3(1), true, partial, nsplit, n,
+                                 R, ldr, x);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }

@@ -32,8 +32,9 @@ __host__ __device__ constexpr int pitch_of(int w) { return w + (w & 1); }
 // Columns missing from the first group.
 __host__ __device__ constexpr int lead_of(int n, int w) { return (n + w - 1) / w * w - n; }
 
-__global__ void k_pack_rinv(const double* __restrict__ X, int64_t ldx, int n, int w, bool from_lower,
-                            double* __restrict__ Rp) {
+__global__ void k_pack_rinv(const double* X, int64_t ldx, int n, int w, bool from_lower,
+                            double* Rp) {
+  grid_chain();
   const int wp = pitch_of(w), lead = lead_of(n, w);
   const int64_t total = (int64_t)NGROUP * n * wp;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -99,8 +100,9 @@ __device__ __forceinline__ void stage_panel(const double* A, int64_t lda, int64_
 // A is deliberately not __restrict__: Q may alias A.
 template <int W>
 __global__ void __launch_bounds__(QT) k_qform_small(const double* A, int64_t lda, int64_t m, int n,
-                                                    const double* __restrict__ Rp, double* Q, int64_t ldq,
+                                                    const double* Rp, double* Q, int64_t ldq,
                                                     int64_t npanels) {
+  grid_chain();
   extern __shared__ double As[];  // [n][PANEL]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int ng = (n + W - 1) / W, lead = lead_of(n, W);
@@ -130,8 +132,9 @@ __global__ void __launch_bounds__(QT) k_qform_small(const double* A, int64_t lda
 // memory ([row][col], odd pitch).
 template <int W, int MAXS>
 __global__ void __launch_bounds__(QT) k_qform_gram_small(const double* A, int64_t lda, int64_t m, int n,
-                                                         const double* __restrict__ Rp, double* Q, int64_t ldq,
-                                                         int64_t rows_per_split, int T, double* __restrict__ partial) {
+                                                         const double* Rp, double* Q, int64_t ldq,
+                                                         int64_t rows_per_split, int T, double* partial) {
+  grid_chain();
   static_assert(QT == GRAM_NT, "the pair list is dealt to this block's threads");
   extern __shared__ double smem[];
   const int pitch = n | 1, ng = (n + W - 1) / W, lead = lead_of(n, W);
@@ -188,7 +191,9 @@ cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const d
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QT, sm);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(npanels, (int64_t)sm_count() * std::max(1, per_sm)));
-  kern<<<(unsigned)grid, QT, sm, s>>>(A, lda, m, n, Rp, Q, ldq, npanels);
+  e = launch_chained(kern, dim3((unsigned)grid), dim3(QT), sm, s, dim3(1), chain_early(2 * grid), A, lda, m, n,
+                     Rp, Q, ldq, npanels);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
@@ -202,7 +207,9 @@ cudaError_t launch_fused(const double* A, int64_t lda, int64_t m, int n, const d
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)((128 + 129) * PANEL * sizeof(double)));
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)g.nsplit, QT, sm, s>>>(A, lda, m, n, Rp, Q, ldq, g.rows_per_split, g.T, partial);
+  e = launch_chained(kern, dim3((unsigned)g.nsplit), dim3(QT), sm, s, dim3(1), chain_early(2 * g.nsplit), A, lda, m,
+                     n, Rp, Q, ldq, g.rows_per_split, g.T, partial);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
@@ -221,7 +228,9 @@ static cudaError_t pack(const double* X, int64_t ldx, int n, bool lower, double*
   if (!w) return cudaErrorInvalidValue;
   const int64_t total = (int64_t)rpack_doubles(n);
   const int grid = (int)std::min<int64_t>(ceil_div(total, 256), 4096);
-  k_pack_rinv<<<grid, 256, 0, s>>>(X, ldx, n, w, lower, Rp);
+  cudaError_t e = launch_chained(k_pack_rinv, dim3((unsigned)grid), dim3(256), 0, s, dim3(1), true, X, ldx, n, w,
+                                 lower, Rp);
+  if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
 }
