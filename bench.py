@@ -470,13 +470,13 @@ def roofline_of(per_stage: dict, m: int, n: int, precision: str, fz: bool, clk: 
     if SLICES[precision] == 0:
         sm_max = clk.get("sm_max_mhz") or 2070.0
         peak = fp64_peak(clk)
+        gram = "k_gram_diag" if n <= 128 else "k_gram_tiles"
         if n <= 256:
-            kern = {"qform1": "k_qform_gram_small" if fz else "k_qform_small", "gram1": "k_gram_tile",
-                    "gram2": "k_gram_tile", "qform2": "k_qform_small"}.get(dom, dom)
+            kern = {"qform1": "k_qform_gram_small" if fz else "k_qform_small", "gram1": gram,
+                    "gram2": gram, "qform2": "k_qform_small"}.get(dom, dom)
         else:
-            kern = {"qform1": "k_gemm_f64", "qform2": "k_gemm_f64", "gram1": "k_gram_tile",
-                    "gram2": "k_gram_tile"}.get(dom, dom)
-        kfile = {"k_gemm_f64": "gemm.cu", "k_gram_tile": "gram.cu"}.get(kern, "qform.cu")
+            kern = {"qform1": "k_gemm_f64", "qform2": "k_gemm_f64", "gram1": gram, "gram2": gram}.get(dom, dom)
+        kfile = {"k_gemm_f64": "gemm.cu", gram: "gram.cu"}.get(kern, "qform.cu")
         note = f"derived FP64 DFMA peak: {FP64_FMA_PER_CLK_PER_SM} FMA/clk/SM x 152 SMs x 2 flops x {sm_max:.0f} MHz"
         bound = "alu"
     else:
@@ -648,7 +648,7 @@ def bench_configs(steps: int, warmup: int, local: int, peaks: dict, clk: dict, s
                     "roofline": {"bound": "alu", "achieved": fl / (ms * 1e-3) / 1e12, "peak": pk, "unit": "TFLOP/s",
                                  "frac": fl / (ms * 1e-3) / 1e12 / pk,
                                  "note": "nominal flops of the whole step over the derived FP64 peak; the step is "
-                                         "latency-bound (two one-CTA CholInv base cases on its critical path)"},
+                                         "latency-bound (two CholInv leaves, a chain of 64 pivots each, on its critical path)"},
                     "errors": dict(errs(hA, Q, R, Ro), oracle_orthogonality=oracle.orthogonality(Qo))})
         ts = []
         for _ in range(5):
