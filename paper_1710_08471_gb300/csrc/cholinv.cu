@@ -178,7 +178,7 @@ cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl,
 // Shift of the shifted CholeskyQR pass: W += s I with
 // s = 11 (m n + n (n+1)) u trace(W), u = 2^-53 (||A||_F^2 = trace(A^T A)).
 // One CTA; the trace is summed in a fixed order.
-__global__ void __launch_bounds__(256) k_add_shift(double* __restrict__ W, int64_t ldw, int n, int64_t m) {
+__global__ void __launch_bounds__(256) k_add_shift(double* W, int64_t ldw, int n, int64_t m) {
   __shared__ double part[256];
   double t = 0.0;
   for (int i = threadIdx.x; i < n; i += 256) t += W[i + (int64_t)i * ldw];

@@ -46,10 +46,12 @@ __device__ __forceinline__ void cp_async_wait() {
 // open with grid_chain(): wait until the predecessor has completed and its
 // writes are visible, then let the successor be set up. Since no grid ends
 // before its own wait, completion stays in stream order, also for what is read
-// and overwritten. Pointers of these kernels carry no __restrict__: a load
-// through the read-only path could be moved above the wait. (us per pass, whole
-// factorizations: least squares of 1024 x 16 79 -> 61, 4096 x 64 202 -> 192,
-// least squares of 131601 x 256 in split precision 2035 -> 2006.)
+// and overwritten. The sources of these kernels hold no __ldg and no
+// __restrict__: the read-only path is for data that stays constant during the
+// kernel's lifetime, which begins before the wait, and such a load could be
+// moved above it. (us per pass, whole factorizations: least squares of
+// 1024 x 16 79 -> 61, 4096 x 64 202 -> 192, least squares of 131601 x 256 in
+// split precision 2035 -> 2006.)
 __device__ __forceinline__ void grid_chain() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

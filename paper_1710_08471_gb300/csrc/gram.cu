@@ -42,8 +42,8 @@ static __device__ __align__(256) double g_noalloc_scratch[NOALLOC_DOUBLES];
 constexpr int NT = GRAM_NT;
 
 // Rows [r0, r1) of columns c0 .. c0 + w - 1 into X[row][column], zeros past r1.
-__device__ __forceinline__ void load_chunk(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int c0,
-                                           int w, double* X, int pitch) {
+__device__ __forceinline__ void load_chunk(const double* A, int64_t lda, int64_t r0, int64_t r1, int c0, int w, double* X,
+                                           int pitch) {
   const int kk = threadIdx.x % KC;
   const int64_t row = r0 + kk;
   const bool ok = row < r1;
@@ -54,8 +54,8 @@ __device__ __forceinline__ void load_chunk(const double* __restrict__ A, int64_t
 
 // One diagonal tile of width w at column c0 over rows [r0, r1).
 template <int MAXS>
-__device__ __forceinline__ void diag_item(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int c0, int w,
-                                          double* smem, double* __restrict__ out, int T) {
+__device__ __forceinline__ void diag_item(const double* A, int64_t lda, int64_t r0, int64_t r1, int c0, int w,
+                                          double* smem, double* out, int T) {
   const int pitch = w | 1;
   GramPairs<MAXS> pairs;
   pairs.init(threadIdx.x, w);
@@ -81,8 +81,8 @@ __device__ __forceinline__ void diag_item(const double* __restrict__ A, int64_t 
 // (wJ <= T) over rows [r0, r1): lane column i = t % T of the first block,
 // columns t / T, t / T + 2, ... of the second.
 template <int S>
-__device__ __forceinline__ void off_item(const double* __restrict__ A, int64_t lda, int64_t r0, int64_t r1, int cI, int cJ,
-                                         int wJ, double* smem, double* __restrict__ out, int T) {
+__device__ __forceinline__ void off_item(const double* A, int64_t lda, int64_t r0, int64_t r1, int cI, int cJ,
+                                         int wJ, double* smem, double* out, int T) {
   const int t = threadIdx.x, pitch = T | 1, i = t % T, jh = t / T;
   const bool live = jh < 2;  // whole warps: T is a multiple of 16
   double acc[S];
@@ -140,8 +140,8 @@ __global__ void __launch_bounds__(NT, MAXS <= 8 ? 3 : (MAXS <= 16 ? 2 : 1))
 // Several tiles: blockIdx.y < noff takes an off-diagonal tile, the others two
 // diagonal ones in turn.
 __global__ void __launch_bounds__(NT, 1)
-    k_gram_tiles(const double* __restrict__ A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T, int ntile,
-                 int ntiles_total, double* __restrict__ partial) {
+    k_gram_tiles(const double* A, int64_t lda, int64_t m, int n, int64_t rows_per_split, int T, int ntile,
+                 int ntiles_total, double* partial) {
   extern __shared__ double smem[];
   const int64_t r0 = (int64_t)blockIdx.x * rows_per_split, r1 = min(m, r0 + rows_per_split);
   double* out = partial + (int64_t)blockIdx.x * ntiles_total * (int64_t)(T * T);

@@ -12,10 +12,12 @@
 // Warp v takes groups v and ng - 1 - v, which evens out the warps' work. (Groups
 // of a power of two from column 0 on, as before: at n = 100 the busiest warp
 // had 1.5 times the mean.) R^-1 is pre-packed per group ([group][k][c],
-// c padded to an even count for 16-byte loads) and read through the read-only
-// path as a warp-wide broadcast; the A panel is staged in shared memory as
-// [k][row], which makes both the global loads and the shared loads
-// conflict-free.
+// c padded to an even count for 16-byte loads) and read as a warp-wide
+// broadcast, with ordinary loads: the kernel may be set up while its
+// predecessor still writes R^-1 (grid_chain), and the read-only path is for
+// data that no one writes during the kernel's lifetime. The A panel is staged
+// in shared memory as [k][row], which makes both the global loads and the
+// shared loads conflict-free.
 #include <algorithm>
 
 #include "gram_pairs.cuh"
@@ -49,10 +51,10 @@ __global__ void k_pack_rinv(const double* X, int64_t ldx, int n, int w, bool fro
 }
 
 template <int W>
-__device__ __forceinline__ void load_w(const double* __restrict__ p, double (&r)[W]) {
+__device__ __forceinline__ void load_w(const double* p, double (&r)[W]) {
 #pragma unroll
   for (int c = 0; c < W; c += 2) {
-    const double2 v = __ldg(reinterpret_cast<const double2*>(p + c));
+    const double2 v = *reinterpret_cast<const double2*>(p + c);
     r[c] = v.x;
     if (c + 1 < W) r[c + 1] = v.y;
   }
@@ -61,7 +63,7 @@ __device__ __forceinline__ void load_w(const double* __restrict__ p, double (&r)
 // Computes the W columns of group g for the lane's row of the staged panel.
 template <int W>
 __device__ __forceinline__ void qform_group(const double* As, int lane, int n, int g,
-                                            const double* __restrict__ Rp, double (&acc)[W]) {
+                                            const double* Rp, double (&acc)[W]) {
   constexpr int WP = pitch_of(W);
   const int c0 = g * W - lead_of(n, W);  // negative for a ragged first group
   const double* rp = Rp + (int64_t)g * n * WP;
