@@ -31,7 +31,7 @@
 // produces (TMA), warp 1 issues tcgen05.mma (M = 128, one MMA per A slice and
 // K = 16 step covering all its products), the other warps drain the group
 // accumulators. Gram: 128 x 64 tiles, one accumulator buffer; Q-form: the same
-// or 128 x 32 tiles with two (oz_qform_shape). All waits are bounded; a timeout
+// or 128 x 32 tiles with two (oz_qform_wide). All waits are bounded; a timeout
 // sets the status word and the CTA unwinds.
 #include <cuda.h>
 
@@ -299,25 +299,6 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
-// The same box into this CTA and its cluster peer, at the same shared-memory
-// offset, signalling the barrier at the same offset in each.
-__device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2,
-                                                 int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-      "[%1, {%3, %4, %5, %6}], [%2], %7;" ::"r"(smem_u32(dst)),
-      "l"(map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "h"((uint16_t)3)
-      : "memory");
-}
-__device__ __forceinline__ void pair_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t pair_rank() {
-  uint32_t r;
-  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
 // MN-major operand (the Q-form's X tile, [k][m] rows of 64 m-values): 128-byte
 // swizzle, 64-element atoms along M 8192 bytes apart (the two TMA boxes), 8-row
 // groups along K 1024 bytes apart; 16 k further is 2048 bytes.
@@ -340,14 +321,6 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
-// The same arrival on the barrier at this offset in both CTAs of the pair.
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -361,7 +334,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
 
 enum { OZ_GRAM = 0, OZ_QFORM = 1 };
 
-// Tile shapes. 128 x 64 tiles (the Gram, and the Q-form where oz_qform_shape
+// Tile shapes. 128 x 64 tiles (the Gram, and the Q-form where oz_qform_wide
 // says so) reuse their operands more; the S group accumulators take 64 S <= 448
 // TMEM columns, one buffer. 128 x 32 tiles have two accumulator buffers (2 x 32
 // S <= 448 columns). The Q-form has 16 epilogue warps, since its epilogue (S
@@ -543,20 +516,14 @@ __device__ __forceinline__ void oz_drain_group(uint32_t ta, long long* X, long l
   }
 }
 
-// Walks a unit's items. The Q-form's items are consecutive, so the row tile
+// Walks a CTA's items. The Q-form's items are consecutive, so the row tile
 // and column tile advance by a counter instead of a 64-bit division per item
-// (which the single MMA-issuing thread would pay between items). BN is the
-// unit's column tile, joff this CTA's part of it.
+// (which the MMA-issuing warp would pay between items).
 template <int MODE, int BN>
 struct OzCursor {
   int64_t rt = 0;  // Q-form: row tile
   int jt = 0;      // Q-form: column tile
-  int64_t unit = 0, units = 1;
-  int joff = 0;
-  __device__ __forceinline__ void init(const OzParams& p, int64_t it0, int64_t u, int64_t us, int jo) {
-    unit = u;
-    units = us;
-    joff = jo;
+  __device__ __forceinline__ void init(const OzParams& p, int64_t it0) {
     if (MODE == OZ_QFORM) {
       rt = it0 / p.ntile_j;
       jt = (int)(it0 - rt * p.ntile_j);
@@ -570,8 +537,8 @@ struct OzCursor {
   }
   __device__ __forceinline__ OzItem item(const OzParams& p, int64_t it) const {
     OzItem w;
-    if (MODE == OZ_GRAM) {  // dealt round-robin: the unit's it-th item
-      w = oz_item<MODE, BN>(p, unit + it * units);
+    if (MODE == OZ_GRAM) {  // dealt round-robin: the CTA's it-th item
+      w = oz_item<MODE, BN>(p, blockIdx.x + it * gridDim.x);
     } else {
       w.j0 = (int64_t)BN * jt;
       w.i0 = (int64_t)OZ_BM * rt;
@@ -579,7 +546,6 @@ struct OzCursor {
       w.split = 0;
       w.nk = oz_qform_nk<BN>(w.j0, p.n);
     }
-    w.j0 += joff;
     return w;
   }
 };
@@ -591,16 +557,7 @@ struct OzCursor {
 // epilogue drains a group as soon as its last product is done and the MMAs
 // overwrite it only after that drain. Warp w of the epilogue reads TMEM lanes
 // 32 (w % 4) .. +31 (its rows) and one column slice of each group.
-//
-// PAIR: a cluster of two CTAs takes one 128-row tile and two neighbouring
-// column tiles of the same contraction range. Both need the same A slices, so
-// each CTA loads half of every slice and multicasts it to both: the A traffic
-// from L2 halves. Alone, a Q-form CTA takes 112 KB of A and 28 KB of B per
-// K-block of 64, for 2300 clocks of MMAs: 60 bytes per clock per SM, more than
-// L2 delivers to all SMs (ms per Q-form, alone and in pairs: 2^23 x 128 9.4 and
-// 7.8, 2^21 x 512 19.6 and 17.2). A Gram CTA takes 44 bytes per clock and gains
-// less (2^23 x 128: 4.66 and 4.46).
-template <int S, int MODE, int BN, int EPI, int NGRP, bool PAIR>
+template <int S, int MODE, int BN, int EPI, int NGRP>
 __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
     k_ozaki_gemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tB, OzParams p) {
   using C = OzCfg<S, MODE, BN, EPI, NGRP>;
@@ -630,15 +587,11 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
     for (int c = threadIdx.x; c < p.n; c += blockDim.x) s_key[c] = 0u;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Work is dealt to units: single CTAs, or pairs, which take column tiles of BNU
-  constexpr int BNU = PAIR ? 2 * BN : BN;
-  const uint32_t rank = PAIR ? pair_rank() : 0;
-  const int64_t unit = PAIR ? blockIdx.x >> 1 : blockIdx.x, units = PAIR ? gridDim.x >> 1 : gridDim.x;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NA; ++i) {
       mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], PAIR ? 2 : 1);  // a slot is free once both CTAs have read it
+      mbar_init(&aempty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&bfull[i], 1);
@@ -658,10 +611,6 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  if (PAIR) {  // the peer's barriers exist before anything arrives on them
-    __syncwarp();
-    pair_sync();
-  }
   asm volatile("tcgen05.fence::after_thread_sync;");
   const uint32_t tmem = *tmem_slot;
   // Gram items are dealt round-robin (the CTA's k-th item is blockIdx.x + k
@@ -669,9 +618,9 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
   // row ranges and read each slice K-block from DRAM once between them, the
   // others finding it in L2. Q-form items go in cost-balanced contiguous
   // ranges (oz_range_begin).
-  const int64_t it_begin = MODE == OZ_GRAM ? 0 : oz_range_begin<MODE, BNU>(p, unit, units);
-  const int64_t it_end = MODE == OZ_GRAM ? (p.nitems > unit ? (p.nitems - unit + units - 1) / units : 0)
-                                         : oz_range_begin<MODE, BNU>(p, unit + 1, units);
+  const int64_t it_begin = MODE == OZ_GRAM ? 0 : oz_range_begin<MODE, BN>(p, blockIdx.x, gridDim.x);
+  const int64_t it_end = MODE == OZ_GRAM ? (p.nitems - blockIdx.x + gridDim.x - 1) / gridDim.x  // grid <= nitems
+                                         : oz_range_begin<MODE, BN>(p, blockIdx.x + 1, gridDim.x);
 
   // Ring positions run on across items: A slot and its phase parity, B buffer
   // and its parity. The issuing warps keep their loops short (no divisions,
@@ -685,8 +634,8 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
       int alast[NA], blast[2];                   // parity of each slot's last fill (-1: none)
       for (int i = 0; i < NA; ++i) alast[i] = -1;
       blast[0] = blast[1] = -1;
-      OzCursor<MODE, BNU> cur;
-      cur.init(p, it_begin, unit, units, (int)rank * BN);
+      OzCursor<MODE, BN> cur;
+      cur.init(p, it_begin);
       for (int64_t it = it_begin; it < it_end && ok; ++it, cur.next(p)) {
         const OzItem w = cur.item(p, it);
         for (int kb = 0; kb < w.nk; ++kb) {
@@ -706,13 +655,7 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
             if (awrapped && !(ok = mbar_wait(&aempty[slot], aph ^ 1u, p.st))) break;
             mbar_expect_tx(&afull[slot], A_BYTES);
             alast[slot] = (int)aph;
-            if (PAIR) {  // this CTA's half of the slice (64 columns of X, or 64 of its rows), for both
-              uint8_t* dst = sA + slot * A_BYTES + rank * (A_BYTES / 2);
-              if (MODE == OZ_GRAM)
-                tma_load_4d_pair(dst, &tB, &afull[slot], 0, (int)w.i0 + 64 * (int)rank, k0 >> 6, s);
-              else
-                tma_load_4d_pair(dst, &tA, &afull[slot], 0, k0, (int)(w.i0 >> 6) + (int)rank, s);
-            } else if (MODE == OZ_GRAM) {
+            if (MODE == OZ_GRAM) {
               tma_load_4d(sA + slot * A_BYTES, &tA, &afull[slot], 0, (int)w.i0, k0 >> 6, s);
             } else {  // X from its column slices: two boxes of 64 rows (m) x 64 columns (k)
               const int kb = (int)(w.i0 >> 6);
@@ -732,11 +675,6 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
           }
         }
       }
-      // A pair's slots also receive the peer's arrivals: the last ones come
-      // before this CTA may leave.
-      if (PAIR && ok)
-        for (int i = 0; i < NA && ok; ++i)
-          if (alast[i] >= 0) ok = mbar_wait(&aempty[i], (uint32_t)alast[i], p.st);
       if (!ok) {
         report_timeout(p.st);
         // wait for the copies still in flight: the last issued fill of every slot
@@ -765,8 +703,8 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
       uint32_t aph = 0, bph = 0;
       int64_t gc = 0;            // chunks issued
       int64_t used0 = 0, used1 = 0;  // two epilogue groups: chunks issued into buffer 0, 1
-      OzCursor<MODE, BNU> cur;
-      cur.init(p, it_begin, unit, units, (int)rank * BN);
+      OzCursor<MODE, BN> cur;
+      cur.init(p, it_begin);
       for (int64_t it = it_begin; it < it_end && ok; ++it, cur.next(p)) {
         const OzItem w = cur.item(p, it);
         const int par_it = (int)((it - it_begin) & 1);
@@ -823,10 +761,7 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
               t0 += nt;
             }
             if (!ok) break;
-            if (el) {
-              if (PAIR) mma_commit_pair(&aempty[slot]);
-              else mma_commit(&aempty[slot]);
-            }
+            if (el) mma_commit(&aempty[slot]);
             // every product of group s is issued; the narrow Q-form's epilogue waits on groups 3 and S-1 only
             if (last && (MODE == OZ_GRAM || CPT != 8 || s == 3 || s == S - 1) && el) mma_commit(&accfull[ab * S + s]);
             if (++slot == NA) {
@@ -857,8 +792,8 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
     const int cs = (ew % (EPI / NGRP)) >> 2;            // column slice of each accumulator
     bool ok = true;
     int64_t gc = 0;  // chunks drained (by this group)
-    OzCursor<MODE, BNU> cur;
-    cur.init(p, it_begin, unit, units, (int)rank * BN);
+    OzCursor<MODE, BN> cur;
+    cur.init(p, it_begin);
     for (int64_t it = it_begin; it < it_end && ok; ++it, cur.next(p)) {
       if (NGRP == 2 && (int)((it - it_begin) & 1) != grp) continue;
       const OzItem w = cur.item(p, it);
@@ -1005,12 +940,6 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
   }
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
-  // neither CTA's shared memory goes away while the peer may still write to it
-  // or arrive on its barriers (every wait above is bounded, so both get here)
-  if (PAIR) {
-    __syncwarp();
-    pair_sync();
-  }
   if (fuse_cmax)
     for (int c = threadIdx.x; c < p.n; c += blockDim.x)
       if (s_key[c] != 0u) atomicMax(p.cmax + c, oz_key_bits(s_key[c]));
@@ -1130,28 +1059,16 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-template <int S, int MODE, int BN, int EPI, int NGRP, bool PAIR>
+template <int S, int MODE, int BN, int EPI, int NGRP>
 cudaError_t launch_oz(const CUtensorMap& a, const CUtensorMap& b, const OzParams& p, int64_t sms, cudaStream_t s) {
   using Cfg = OzCfg<S, MODE, BN, EPI, NGRP>;
   constexpr size_t SMEM = Cfg::SMEM;
   static_assert(MODE != OZ_QFORM || Cfg::KEYS >= OZ_CMAX_N, "column max keys");
   static_assert(SMEM <= 227 * 1024, "shared memory per CTA");
-  auto kern = k_ozaki_gemm<S, MODE, BN, EPI, NGRP, PAIR>;
+  auto kern = k_ozaki_gemm<S, MODE, BN, EPI, NGRP>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
   if (e != cudaSuccess) return e;
-  constexpr int CPU = PAIR ? 2 : 1;  // CTAs per unit
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(CPU * std::min<int64_t>(p.nitems, std::max<int64_t>(1, sms / CPU))));
-  cfg.blockDim = dim3(Cfg::THREADS);
-  cfg.dynamicSmemBytes = SMEM;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = CPU;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = PAIR ? 1 : 0;
-  if ((e = cudaLaunchKernelEx(&cfg, kern, a, b, p)) != cudaSuccess) return e;
+  kern<<<(unsigned)std::min<int64_t>(p.nitems, sms), Cfg::THREADS, SMEM, s>>>(a, b, p);
   count_launch();
   return cudaGetLastError();
 }
@@ -1178,52 +1095,45 @@ bool ozaki_supported(int n, int S) { return n >= 1 && n <= OZAKI_MAX_N && S >= 6
 namespace {
 constexpr int64_t OZ_MAX_CHUNKS_PER_SPLIT = (1 << 20) / 128;  // fixed-point headroom
 
-// Tiles touching the upper triangle: row blocks of 128, nj column tiles, r per row block.
-int oz_gram_tiles(int nj, int r) {
+// Gram tiles touching the upper triangle.
+int oz_gram_tiles(int n) {
+  constexpr int R = OZ_BM / OZ_GRAM_BN;  // column tiles per 128-row block
+  const int nj = (int)ceil_div(n, OZ_GRAM_BN);
   int t = 0;
-  for (int I = 0; r * I < nj; ++I) t += nj - r * I;
+  for (int I = 0; R * I < nj; ++I) t += nj - R * I;
   return t;
 }
 
-// Pairs of column tiles on two CTAs: where the tiles pair up (a pair with one
-// tile past the last column leaves a CTA idle for its time).
-bool oz_gram_pairs(int n) {
-  const int nj = (int)ceil_div(n, OZ_GRAM_BN), np = (int)ceil_div(n, 2 * OZ_GRAM_BN);
-  return 2.0 * oz_gram_tiles(np, 1) <= 1.15 * oz_gram_tiles(nj, OZ_BM / OZ_GRAM_BN);
-}
-
-// The Q-form's shape: 32-column tiles on single CTAs or on pairs, or 64-column
-// tiles on pairs. A wider tile reuses each A slice more often: per K-block the
-// shared-memory port (128 bytes per clock) serves the MMAs' operands and the
-// incoming slices in 2850 clocks for 32 columns and 4300 for 64; but its
-// accumulators fill TMEM (one buffer), and a ragged last tile costs more. Costs
-// per row tile, in K-blocks plus half a one per tile, of a pair's narrow tiles;
-// singles 1.2 times (their A traffic), wide ones 1.65 times. Measured at 2^27
-// entries, us for both Q-forms, narrow pairs and wide: n = 128 1334, 1406; 200
-// 2463, 2392; 256 1945, 1904; 320 2292, 2723; 512 3281, 2981; 768 4609, 3990.
-enum OzQShape { OZ_Q_SINGLE, OZ_Q_PAIR, OZ_Q_WIDE };
-OzQShape oz_qform_shape(int n) {
-  auto cost = [n](int bn) {
+// Whether the Q-form takes 64-column tiles instead of 32-column ones. A wider
+// tile reuses each A slice more often (per 32 columns and K-block of 64 the
+// CTA takes 84 KB from L2, not 140 KB); but its accumulators fill TMEM (one
+// buffer, so a tile's last drain is not hidden), and a ragged last tile costs
+// more. Costs per row tile in K-blocks of a narrow tile: a quarter per narrow
+// tile beside its K-blocks; 1.55 per K-block of a wide one and one K-block more
+// per tile. Measured at 2^26 entries, us per Q-form, narrow and wide: n = 64 670,
+// 733; 128 714, 750; 160 833, 1224; 200 (2^27 entries) 1094, 1392; 248 1081,
+// 1018; 288 1122, 1176; 384 1364, 1190; 416 1483, 1552; 512 1730, 1590; 640 2289,
+// 1833; 768 3139, 2131; 1024 4523, 2704; of 72 widths and slice counts the rule
+// misses the better one by more than 2% twice (256: 1078, 1124).
+bool oz_qform_wide(int n) {
+  auto cost = [n](int bn, double per_tile) {
     double c = 0.0;
-    for (int j = 0; j < n; j += bn) c += std::min(ceil_div(j + bn, OZ_BK), ceil_div(n, OZ_BK)) + 0.5;
+    for (int j = 0; j < n; j += bn) c += std::min(ceil_div(j + bn, OZ_BK), ceil_div(n, OZ_BK)) + per_tile;
     return c;
   };
-  const double single = 0.6 * cost(OZ_QFORM_BN), pair = cost(2 * OZ_QFORM_BN), wide = 1.65 * cost(2 * OZ_QFORM_BN_WIDE);
-  return wide < pair && wide < single ? OZ_Q_WIDE : (pair <= single ? OZ_Q_PAIR : OZ_Q_SINGLE);
+  return 1.55 * cost(OZ_QFORM_BN_WIDE, 1.0) < cost(OZ_QFORM_BN, 0.25);
 }
 
 // Row ranges of the Gram: its items (ranges x tiles) all cost the same and are
-// dealt to the units (CTAs, or pairs of them) in whole rounds, so the ranges
-// are chosen to fill the rounds: the fewest rounds, up to four, that leave less
-// than 5% of the units idle, or else the count that leaves the fewest. (Two
-// items per CTA whatever the tiles, as before, made three rounds of 2.1 at
-// n = 200 and n = 512, a third of the time idle: 2^21 x 512 15.5 -> 11.1 ms per
-// Gram, 1000037 x 200 with six slices 1.82 -> 1.36.)
+// dealt to the CTAs in whole rounds, so the ranges are chosen to fill the
+// rounds: the fewest rounds, up to four, that leave less than 5% of the CTAs
+// idle, or else the count that leaves the fewest. (Two items per CTA whatever
+// the tiles, as before, made three rounds of 2.1 at n = 200 and n = 512, a third
+// of the time idle: 2^21 x 512 15.5 -> 11.1 ms per Gram, 1000037 x 200 with six
+// slices 1.82 -> 1.36.)
 int64_t oz_split_target(int n) {
-  const bool pair = oz_gram_pairs(n);
-  const int64_t units = std::max<int64_t>(1, sm_count_oz() / (pair ? 2 : 1));
-  const int tiles = pair ? oz_gram_tiles((int)ceil_div(n, 2 * OZ_GRAM_BN), 1)
-                         : oz_gram_tiles((int)ceil_div(n, OZ_GRAM_BN), OZ_BM / OZ_GRAM_BN);
+  const int64_t units = sm_count_oz();
+  const int tiles = oz_gram_tiles(n);
   int64_t best = 1;
   double best_use = 0.0;
   for (int r = 1; r <= 4; ++r) {
@@ -1345,18 +1255,15 @@ cudaError_t ozaki_gram(const OzMaps& maps, int64_t m, int n, int S, const int* c
   p.ldo = n;
   p.st = st;
   p.gate = gate;
-  const bool pair = oz_gram_pairs(n);
-  p.ntile_j = (int)ceil_div(n, pair ? 2 * OZ_GRAM_BN : OZ_GRAM_BN);
-  p.ntiles = oz_gram_tiles(p.ntile_j, pair ? 1 : OZ_BM / OZ_GRAM_BN);
+  p.ntile_j = (int)ceil_div(n, OZ_GRAM_BN);
+  p.ntiles = oz_gram_tiles(n);
   p.nitems = (int64_t)p.ntiles * g.nsplit;
   const CUtensorMap& a = *(const CUtensorMap*)maps.col_a;
   const CUtensorMap& b = *(const CUtensorMap*)maps.col_b;
   const int64_t sms = sm_count_oz();
   constexpr int BN = OZ_GRAM_BN, EPI = OZ_GRAM_EPI, GRP = OZ_GRAM_GRP;
-  cudaError_t e = pair ? (S == 7 ? launch_oz<7, OZ_GRAM, BN, EPI, GRP, true>(a, b, p, sms, s)
-                                 : launch_oz<6, OZ_GRAM, BN, EPI, GRP, true>(a, b, p, sms, s))
-                       : (S == 7 ? launch_oz<7, OZ_GRAM, BN, EPI, GRP, false>(a, b, p, sms, s)
-                                 : launch_oz<6, OZ_GRAM, BN, EPI, GRP, false>(a, b, p, sms, s));
+  cudaError_t e = S == 7 ? launch_oz<7, OZ_GRAM, BN, EPI, GRP>(a, b, p, sms, s)
+                         : launch_oz<6, OZ_GRAM, BN, EPI, GRP>(a, b, p, sms, s);
   if (e != cudaSuccess) return e;
   dim3 rg((unsigned)ceil_div(n, 32), (unsigned)n);
   k_oz_gram_reduce<<<rg, 32 * OZ_RC, 0, s>>>(partial, g.nsplit, n, W, ldw, gate, S);
@@ -1376,10 +1283,8 @@ cudaError_t ozaki_qform(const OzMaps& maps, int64_t m, int n, int S, const int* 
   p.out = Q;
   p.ldo = ldq;
   p.st = st;
-  const OzQShape shape = oz_qform_shape(n);
-  const bool wide = shape == OZ_Q_WIDE, pair = shape != OZ_Q_SINGLE;
-  const int bn = wide ? OZ_QFORM_BN_WIDE : OZ_QFORM_BN;
-  p.ntile_j = (int)ceil_div(n, pair ? 2 * bn : bn);
+  const bool wide = oz_qform_wide(n);
+  p.ntile_j = (int)ceil_div(n, wide ? OZ_QFORM_BN_WIDE : OZ_QFORM_BN);
   p.ntiles = 1;
   p.nitems = (int64_t)p.ntile_j * ceil_div(m, OZ_BM);
   p.gate = gate;
@@ -1388,13 +1293,10 @@ cudaError_t ozaki_qform(const OzMaps& maps, int64_t m, int n, int S, const int* 
   const int64_t sms = sm_count_oz();
   constexpr int BN = OZ_QFORM_BN, BNW = OZ_QFORM_BN_WIDE, EPI = OZ_QFORM_EPI, GRP = OZ_QFORM_GRP;
   if (wide)
-    return S == 7 ? launch_oz<7, OZ_QFORM, BNW, EPI, GRP, true>(a, b, p, sms, s)
-                  : launch_oz<6, OZ_QFORM, BNW, EPI, GRP, true>(a, b, p, sms, s);
-  if (pair)
-    return S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s)
-                  : launch_oz<6, OZ_QFORM, BN, EPI, GRP, true>(a, b, p, sms, s);
-  return S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s)
-                : launch_oz<6, OZ_QFORM, BN, EPI, GRP, false>(a, b, p, sms, s);
+    return S == 7 ? launch_oz<7, OZ_QFORM, BNW, EPI, GRP>(a, b, p, sms, s)
+                  : launch_oz<6, OZ_QFORM, BNW, EPI, GRP>(a, b, p, sms, s);
+  return S == 7 ? launch_oz<7, OZ_QFORM, BN, EPI, GRP>(a, b, p, sms, s)
+                : launch_oz<6, OZ_QFORM, BN, EPI, GRP>(a, b, p, sms, s);
 }
 
 cudaError_t ozaki_route(const int* cexp, const double* W, int64_t ldw, int n, int64_t m, int* gate, bool keep,
