@@ -181,20 +181,29 @@ int sm_count() {
   return sms;
 }
 
+// A grid that is set up early asks for more than half of an SM's shared memory,
+// so that no two of its CTAs share an SM: placed while the predecessor still
+// holds most SMs, they piled up on the others, up to three on one, each with a
+// panel of 70 (n = 128) to 277 us (n = 256). us per factorization: 2432 x 256
+// 2407 -> 1382, 512 x 256 2207 -> 1183, 2000 x 200 1399 -> 928; 1024 x 16 and
+// 4096 x 64 unchanged.
+constexpr int QFORM_ALONE_SMEM = 118 * 1024;
+static_assert(QFORM_ALONE_SMEM >= 256 * PANEL * (int)sizeof(double), "the widest matrix's panel");
+
 template <int W>
 cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q, int64_t ldq,
                          cudaStream_t s) {
   const size_t sm = (size_t)n * PANEL * sizeof(double);
   auto kern = k_qform_small<W>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(16 * W * PANEL * sizeof(double)));  // of the widest matrix
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, QFORM_ALONE_SMEM);
   if (e != cudaSuccess) return e;
   const int64_t npanels = ceil_div(m, PANEL);
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QT, sm);
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(npanels, (int64_t)sm_count() * std::max(1, per_sm)));
-  e = launch_chained(kern, dim3((unsigned)grid), dim3(QT), sm, s, dim3(1), chain_early(2 * grid), A, lda, m, n,
-                     Rp, Q, ldq, npanels);
+  const bool early = chain_early(2 * grid);
+  e = launch_chained(kern, dim3((unsigned)grid), dim3(QT), early ? (size_t)QFORM_ALONE_SMEM : sm, s, dim3(1), early, A,
+                     lda, m, n, Rp, Q, ldq, npanels);
   if (e != cudaSuccess) return e;
   count_launch();
   return cudaGetLastError();
