@@ -169,6 +169,14 @@ cqr2_status_t cqr2_lstsq_rows(cqr2_plan_t plan, int64_t m, const double* dA, int
 cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t plan, int32_t ctas_per_sm);
 cqr2_status_t cqr2_plan_set_fused(cqr2_plan_t plan, int32_t fused);
 
+/* Whether calls of other plans run on the GPU beside this plan's (0, the
+ * default, or 1). Launch shapes are otherwise chosen for a call that has the
+ * GPU to itself; with 1 they let the streams' kernels interleave, which lowers
+ * the latency of many calls at a time and slows one alone (the smallest most). The result
+ * is the same up to rounding. Not for use while the plan's stream has a call in
+ * flight. */
+cqr2_status_t cqr2_plan_set_shared(cqr2_plan_t plan, int32_t shared);
+
 /* Inverse depth (the paper's alternative of triangular inverted blocks,
  * Section III-A "3D-CQR2", and its InverseDepth parameter, Section IV): with
  * depth d > 0 the top d halvings of CholInv (Algorithm 1) do not form the

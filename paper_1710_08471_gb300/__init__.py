@@ -240,6 +240,10 @@ def cqr2_plan_set_gram_ctas(plan, ctas_per_sm: int) -> None:
     N.check(N.load().cqr2_plan_set_gram_ctas(plan, ctas_per_sm), "cqr2_plan_set_gram_ctas")
 
 
+def cqr2_plan_set_shared(plan, shared: bool) -> None:
+    N.check(N.load().cqr2_plan_set_shared(plan, 1 if shared else 0), "cqr2_plan_set_shared")
+
+
 def cqr2_plan_set_fused(plan, fused: bool) -> None:
     N.check(N.load().cqr2_plan_set_fused(plan, 1 if fused else 0), "cqr2_plan_set_fused")
 
@@ -399,6 +403,10 @@ class Plan:
 
     def set_inverse_depth(self, depth: int) -> None:
         cqr2_plan_set_inverse_depth(self.handle, depth)
+
+    def set_shared(self, shared: bool) -> None:
+        """Other plans' calls run on the GPU beside this plan's."""
+        cqr2_plan_set_shared(self.handle, shared)
 
     def set_fused(self, fused: bool) -> None:
         cqr2_plan_set_fused(self.handle, fused)

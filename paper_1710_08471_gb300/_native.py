@@ -69,6 +69,7 @@ SIGNATURES = {
     "cqr2_plan_split_slices": (C.c_int, [_P, C.POINTER(C.c_int32)]),
     "cqr2_plan_set_panel_width": (C.c_int, [_P, _I64]),
     "cqr2_plan_set_gram_ctas": (C.c_int, [_P, C.c_int32]),
+    "cqr2_plan_set_shared": (C.c_int, [_P, C.c_int32]),
     "cqr2_plan_set_fused": (C.c_int, [_P, C.c_int32]),
     "cqr2_plan_set_inverse_depth": (C.c_int, [_P, C.c_int32]),
     "cqr2_selftest_wait_timeout": (C.c_int, [C.c_int64, _P]),

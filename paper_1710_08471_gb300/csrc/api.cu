@@ -43,6 +43,7 @@ struct cqr2_plan_st {
   bool small = false;  // n <= 256: panel Q-form kernel, Q1 staged in the output Q
   bool fused = false;  // CQR2_FUSED requested and n small enough to fuse
   int64_t gemv_nsplit = 0;
+  bool shared = false;  // other calls run beside this plan's (cqr2_plan_set_shared)
   // device workspace (one allocation)
   char* ws = nullptr;
   size_t ws_bytes = 0;
@@ -112,6 +113,8 @@ namespace {
 
 constexpr int GRAM_CPS_MAX = 8;
 
+Lane lane(const cqr2_plan_st* p) { return Lane(p->stream, p->shared); }
+
 #define TRY(call)                             \
   do {                                        \
     cudaError_t e_ = (call);                  \
@@ -122,7 +125,7 @@ constexpr int GRAM_CPS_MAX = 8;
 // R = R' R0 of the shifted variant); op(A) = A^T when A holds a lower
 // Cholesky factor.
 cudaError_t r_product(cqr2_plan_st* p, int n, const double* A, int64_t lda, bool a_trans, const double* B,
-                      int64_t ldb, double* C, int64_t ldc, cudaStream_t s) {
+                      int64_t ldb, double* C, int64_t ldc, Lane s) {
   if (n <= TRMM_SMALL_MAX) return trmm_upper_small(n, A, lda, a_trans, B, ldb, C, ldc, s);
   return gemm_f64(n, n, n, 1.0, A, lda, B, ldb, 0.0, C, ldc,
                   (a_trans ? GEMM_TA : 0u) | GEMM_A_UPPER | GEMM_B_UPPER | GEMM_C_UPPER | GEMM_BETA0, s);
@@ -192,7 +195,7 @@ cudaError_t hx_wait_input(cqr2_plan_st* p, cudaStream_t s) {
 // [L, Y] = CholInv(W) of the plan's pass, with the plan's inverse depth.
 // [L, Y] = CholInv(W) into the plan's L and Y, and, when given, R = L^T into Rt
 // (ld n) and the Q-form's packed R^-1 into Rp.
-cudaError_t plan_cholinv(cqr2_plan_st* p, int pass, cudaStream_t s, double* Rt = nullptr, double* Rp = nullptr) {
+cudaError_t plan_cholinv(cqr2_plan_st* p, int pass, Lane s, double* Rt = nullptr, double* Rp = nullptr) {
   const int n = (int)p->n;
   if (p->inv_depth > 0) {
     cudaError_t e = cholinv_depth(n, p->W, n, p->L, n, p->Y, n, p->Wk, p->U, p->Tsolve, p->ldt, p->st, pass,
@@ -207,7 +210,7 @@ cudaError_t plan_cholinv(cqr2_plan_st* p, int pass, cudaStream_t s, double* Rt =
 // X = B R^-1 = B L^-T (general path, rows x n): one triangular multiply by
 // the whole inverse, or block forward substitution at inverse depth d > 0.
 cudaError_t plan_apply_rinv(cqr2_plan_st* p, int64_t rows, const double* B, int64_t ldb, double* X, int64_t ldx,
-                            cudaStream_t s) {
+                            Lane s) {
   const int n = (int)p->n;
   if (p->inv_depth > 0)
     return right_solve(rows, n, B, ldb, X, ldx, p->L, n, p->Y, n, p->inv_depth, p->Tsolve, p->ldt, s);
@@ -237,8 +240,8 @@ namespace {
 cqr2_status_t set_rows(cqr2_plan_st* p, int64_t m) {
   if (m < p->n || m > p->m) return CQR2_ERR_INVALID_ARG;
   if (m == p->cm) return CQR2_OK;
-  p->g = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps);
-  p->gf = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps, QFORM_PANEL);
+  p->g = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps, 4, p->shared);
+  p->gf = gram_geometry(m, (int)p->n, p->gram_cap, p->gram_cps, QFORM_PANEL, p->shared);
   p->gemv_nsplit = gemv_splits(m, (int)p->n);
   if (p->oz_S && ozaki_make_maps(p->oz_maps, m, (int)p->n, p->oz_Scap, p->oz_planes, p->oz_rinv) != cudaSuccess) {
     p->cm = 0;
@@ -263,7 +266,7 @@ cqr2_status_t factor_impl_ozaki(cqr2_plan_st* p, const double* dA, int64_t lda, 
                                 int64_t ldr, int pass_base = 0) {
   const int n = (int)p->n, S = p->oz_S;
   const int64_t m = p->cm;
-  cudaStream_t s = p->stream;
+  const Lane s = lane(p);
   const bool route = S == 6;
   const int* gate = route ? p->oz_gate : nullptr;
   if (!pass_base) TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s));
@@ -343,7 +346,7 @@ cqr2_status_t factor_impl(cqr2_plan_st* p, const double* dA, int64_t lda, double
                           int64_t ldr, int pass_base = 0) {
   if (p->oz_S) return factor_impl_ozaki(p, dA, lda, dQ, ldq, dR, ldr, pass_base);
   const int n = (int)p->n;
-  cudaStream_t s = p->stream;
+  const Lane s = lane(p);
   if (!pass_base) TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s));
   // ---- pass 1: W1 = A^T A, [L1, Y1] = CholInv(W1)
   {
@@ -357,7 +360,7 @@ cqr2_status_t factor_impl(cqr2_plan_st* p, const double* dA, int64_t lda, double
         const int64_t r0 = hx_row(p->cm, b), r1 = hx_row(p->cm, b + 1);
         TRY(cudaStreamWaitEvent(s, p->hx_ev[b], 0));
         if (r1 <= r0) continue;
-        const GramGeom gr = gram_geometry(r1 - r0, n, p->hx_cap, p->gram_cps);
+        const GramGeom gr = gram_geometry(r1 - r0, n, p->hx_cap, p->gram_cps, 4, p->shared);
         TRY(gram_partials(dA + r0, lda, r1 - r0, n, gr, p->hx_partial + used * per_split, s));
         used += gr.nsplit;
       }
@@ -455,7 +458,7 @@ cqr2_status_t factor_any(cqr2_plan_st* p, const double* dA, int64_t lda, double*
 cqr2_status_t factor_panels(cqr2_plan_st* p, const double* dA, int64_t lda, double* dQ, int64_t ldq, double* dR,
                             int64_t ldr) {
   const int64_t n = p->n, m = p->cm, b = p->panel_b;
-  cudaStream_t s = p->stream;
+  const Lane s = lane(p);
   TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s));
   TRY(hx_wait_input(p, s));
   // R's strictly lower part stays zero; its blocks are written panel by panel
@@ -488,7 +491,7 @@ cqr2_status_t factor_any(cqr2_plan_st* p, const double* dA, int64_t lda, double*
   if (!(p->flags & CQR2_SHIFTED)) return factor_impl(p, dA, lda, dQ, ldq, dR, ldr, 0);
   const int n = (int)p->n;
   const int64_t m = p->cm;
-  cudaStream_t s = p->stream;
+  const Lane s = lane(p);
   TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), s));
   TRY(hx_wait_input(p, s));
   {
@@ -762,14 +765,9 @@ cqr2_status_t cqr2_plan_set_panel_width(cqr2_plan_t p, int64_t b) {
     p->pan_C = nullptr;
     return r;
   }
-  if (p->gexec) {  // a captured graph of the unpaneled sequence no longer applies
-    cudaGraphExecDestroy(p->gexec);
-    cudaGraphDestroy(p->graph);
-    p->gexec = nullptr;
-    p->graph = nullptr;
-  }
   p->panel_b = b;
-  return CQR2_OK;
+  // the panels' plans too; a captured graph of the unpaneled sequence goes
+  return cqr2_plan_set_shared(p, p->shared);
 }
 
 cqr2_status_t cqr2_plan_split_slices(cqr2_plan_t plan, int32_t* slices) {
@@ -842,6 +840,19 @@ cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t p, int32_t ctas_per_sm) {
   if (!p || ctas_per_sm < 1 || ctas_per_sm > GRAM_CPS_MAX) return CQR2_ERR_INVALID_ARG;
   p->gram_cps = ctas_per_sm;
   p->cm = 0;  // recompute the geometry on the next call
+  if (p->gexec) cudaGraphExecDestroy(p->gexec);
+  if (p->graph) cudaGraphDestroy(p->graph);
+  p->gexec = nullptr;
+  p->graph = nullptr;
+  return CQR2_OK;
+}
+
+cqr2_status_t cqr2_plan_set_shared(cqr2_plan_t p, int32_t shared) {
+  if (!p) return CQR2_ERR_INVALID_ARG;
+  p->shared = shared != 0;
+  p->cm = 0;  // recompute the geometry on the next call
+  if (p->pan_full) cqr2_plan_set_shared(p->pan_full, shared);
+  if (p->pan_tail) cqr2_plan_set_shared(p->pan_tail, shared);
   if (p->gexec) cudaGraphExecDestroy(p->gexec);
   if (p->graph) cudaGraphDestroy(p->graph);
   p->gexec = nullptr;
@@ -936,8 +947,8 @@ cqr2_status_t cqr2_lstsq_rows(cqr2_plan_t p, int64_t m, const double* dA, int64_
   if ((r = factor_any(p, dA, lda, dQ, ldq, R, ldR)) != CQR2_OK) return r;
   {
     Stage st(p, CQR2_STAGE_LSTSQ);
-    TRY(gemv_t_partials(dQ, ldq, p->cm, (int)p->n, db, p->gemv_nsplit, p->lspart, p->stream));
-    TRY(lstsq_solve(p->lspart, p->gemv_nsplit, (int)p->n, R, ldR, dx, p->stream));
+    TRY(gemv_t_partials(dQ, ldq, p->cm, (int)p->n, db, p->gemv_nsplit, p->lspart, lane(p)));
+    TRY(lstsq_solve(p->lspart, p->gemv_nsplit, (int)p->n, R, ldR, dx, lane(p)));
   }
   if (info) return read_info(p, info);
   return CQR2_OK;
@@ -956,8 +967,8 @@ cqr2_status_t cqr2_syrk(cqr2_plan_t p, const double* dA, int64_t lda, double* dW
     TRY(ozaki_gram(p->oz_maps, p->cm, n, p->oz_S, p->oz_cexp, p->oz_partial, p->oz_cap, dW, ldw, p->st, p->stream));
     return CQR2_OK;
   }
-  TRY(gram_partials(dA, lda, p->cm, (int)p->n, p->g, p->partial, p->stream));
-  TRY(gram_reduce(p->partial, p->g, (int)p->n, dW, ldw, p->stream));
+  TRY(gram_partials(dA, lda, p->cm, (int)p->n, p->g, p->partial, lane(p)));
+  TRY(gram_reduce(p->partial, p->g, (int)p->n, dW, ldw, lane(p)));
   return CQR2_OK;
 }
 
@@ -968,7 +979,7 @@ cqr2_status_t cqr2_cholinv(cqr2_plan_t p, const double* dW, int64_t ldw, double*
   cqr2_status_t r = check_device(p);
   if (r != CQR2_OK) return r;
   TRY(cudaMemsetAsync(p->st, 0, sizeof(DevStatus), p->stream));
-  TRY(cholinv((int)p->n, dW, ldw, dL, ldl, dY, ldy, p->Wk, p->U, p->st, 1, p->stream));
+  TRY(cholinv((int)p->n, dW, ldw, dL, ldl, dY, ldy, p->Wk, p->U, p->st, 1, lane(p)));
   if (info) return read_info(p, info);
   return CQR2_OK;
 }
@@ -989,10 +1000,10 @@ cqr2_status_t cqr2_qform(cqr2_plan_t p, const double* dA, int64_t lda, const dou
     TRY(ozaki_slice_rinv(dRinv, ldri, n, p->oz_S, true, p->oz_cexp, p->oz_rinv, p->oz_fexp, p->stream));
     TRY(ozaki_qform(p->oz_maps, p->cm, n, p->oz_S, p->oz_fexp, dQ, ldq, p->st, p->stream));
   } else if (p->small) {
-    TRY(pack_rinv_from_upper(dRinv, ldri, n, p->Rp, p->stream));
-    TRY(qform_small(dA, lda, p->cm, n, p->Rp, dQ, ldq, p->stream));
+    TRY(pack_rinv_from_upper(dRinv, ldri, n, p->Rp, lane(p)));
+    TRY(qform_small(dA, lda, p->cm, n, p->Rp, dQ, ldq, lane(p)));
   } else {
-    TRY(gemm_f64(p->cm, n, n, 1.0, dA, lda, dRinv, ldri, 0.0, dQ, ldq, GEMM_B_UPPER | GEMM_BETA0, p->stream));
+    TRY(gemm_f64(p->cm, n, n, 1.0, dA, lda, dRinv, ldri, 0.0, dQ, ldq, GEMM_B_UPPER | GEMM_BETA0, lane(p)));
   }
   return CQR2_OK;
 }
@@ -1004,7 +1015,7 @@ cqr2_status_t cqr2_trmm_upper(cqr2_plan_t p, const double* dR2, int64_t ld2, con
   cqr2_status_t r = check_device(p);
   if (r != CQR2_OK) return r;
   const int n = (int)p->n;
-  TRY(r_product(p, n, dR2, ld2, false, dR1, ld1, dR, ldr, p->stream));
+  TRY(r_product(p, n, dR2, ld2, false, dR1, ld1, dR, ldr, lane(p)));
   return CQR2_OK;
 }
 

@@ -42,7 +42,7 @@ __global__ void k_copy_upper(const double* X, int64_t ldx, int n, double* R, int
 }
 
 cudaError_t rec(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, double* Y, int64_t ldy, double* U,
-                int64_t ldu, DevStatus* st, int pass, long long off, cudaStream_t s) {
+                int64_t ldu, DevStatus* st, int pass, long long off, Lane s) {
   if (n <= CHOLINV_LEAF) return cholinv_leaf(n, Wk, ldk, L, ldl, Y, ldy, nullptr, 0, nullptr, 0, st, pass, off, s);
   const int n1 = NB * (int)ceil_div(n, 2 * NB);
   const int n2 = n - n1;
@@ -73,7 +73,7 @@ cudaError_t rec(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, double* 
 // substitution through the diagonal blocks' inverses and leave Y21 zero.
 cudaError_t rec_depth(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, double* Y, int64_t ldy, double* U,
                       int64_t ldu, double* T, int64_t ldt, DevStatus* st, int pass, long long off, int depth,
-                      cudaStream_t s) {
+                      Lane s) {
   if (depth <= 0 || n <= NB) return rec(n, Wk, ldk, L, ldl, Y, ldy, U, ldu, st, pass, off, s);
   const int n1 = NB * (int)ceil_div(n, 2 * NB);
   const int n2 = n - n1;
@@ -97,7 +97,7 @@ cudaError_t rec_depth(int n, double* Wk, int64_t ldk, double* L, int64_t ldl, do
 
 cudaError_t right_solve(int64_t M, int N, const double* B, int64_t ldb, double* X, int64_t ldx, const double* L,
                         int64_t ldl, const double* Y, int64_t ldy, int depth, double* T, int64_t ldt,
-                        cudaStream_t s) {
+                        Lane s) {
   cudaError_t e;
   if (M <= 0 || N <= 0) return cudaSuccess;
   if (depth <= 0 || N <= NB) {
@@ -130,7 +130,7 @@ int right_solve_temp_cols(int n) { return n <= NB ? n : NB * (int)ceil_div(n, 2 
 
 cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                           double* work, double* U, double* T, int64_t ldt, DevStatus* st, int pass, int depth,
-                          cudaStream_t s) {
+                          Lane s) {
   if (depth <= 0) return cholinv(n, W, ldw, L, ldl, Y, ldy, work, U, st, pass, s);
   cudaError_t e;
   if ((e = cudaMemcpy2DAsync(work, (size_t)n * sizeof(double), W, (size_t)ldw * sizeof(double),
@@ -146,7 +146,7 @@ cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_
 }
 
 cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
-                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s,
+                    double* work, double* U, DevStatus* st, int pass, Lane s,
                     double* Rt, int64_t ldrt, double* Rp) {
   cudaError_t e;
   if (n <= CHOLINV_LEAF) {
@@ -198,7 +198,7 @@ cudaError_t add_shift(double* W, int64_t ldw, int n, int64_t m, cudaStream_t s) 
   return cudaGetLastError();
 }
 
-cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int64_t ldr, cudaStream_t s) {
+cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int64_t ldr, Lane s) {
   dim3 grid((unsigned)ceil_div(n, 32), (unsigned)ceil_div(n, 32));
   cudaError_t e = launch_chained(k_transpose_lower, grid, dim3(32, 8), 0, s, dim3(1), true, L, ldl, n, R, ldr);
   if (e != cudaSuccess) return e;
@@ -206,7 +206,7 @@ cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int6
   return cudaGetLastError();
 }
 
-cudaError_t copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr, cudaStream_t s) {
+cudaError_t copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr, Lane s) {
   dim3 grid((unsigned)ceil_div(n, 128), (unsigned)n);
   cudaError_t e = launch_chained(k_copy_upper, grid, dim3(128), 0, s, dim3(1), true, X, ldx, n, R, ldr);
   if (e != cudaSuccess) return e;

@@ -540,7 +540,7 @@ static int leaf_ctas(int n) {
 
 cudaError_t cholinv_leaf(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                          double* Rt, int64_t ldrt, double* Rp, int rpw, DevStatus* st, int pass, long long off,
-                         cudaStream_t s) {
+                         Lane s) {
   if (n < 1 || n > CHOLINV_LEAF) return cudaErrorInvalidValue;
   const int C = leaf_ctas(n);
   const size_t sm = leaf_smem(n, C);

@@ -39,6 +39,26 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N));
 }
 
+// The stream a call's kernels go to, and whether other calls' kernels run
+// beside them (cqr2_plan_set_shared). Launch shapes are chosen for a call that
+// has the GPU to itself; a shared lane takes what lets the streams interleave:
+// no grid is set up early (it holds its slots while it waits), no product
+// splits k over a cluster (which starts only where several SMs of a group have
+// room at once), the Gram's ranges and the Q-form's panels go in shorter CTAs
+// (between which the other streams' kernels start; a whole-wave Gram CTA holds
+// its SM for up to 14 ms). Median latency of 500 FP64 least-squares requests at
+// 100/s on 8 slots, three arrival seeds, ms: 15.8, 25.5, 44.8 with the shapes of
+// a call alone and 14.0, 19.9, 40.7 shared; with early set-up 14.0, 22.1, 42.3,
+// with k splits 14.2, 20.9, 41.3, with the Gram in one wave 14.3, 21.5, 40.7, with
+// the Q-form in one wave 13.9, 20.4, 41.3. One request at a time then takes 0.7%
+// longer.
+struct Lane {
+  cudaStream_t s;
+  bool shared;
+  Lane(cudaStream_t s_, bool shared_ = false) : s(s_), shared(shared_) {}
+  operator cudaStream_t() const { return s; }
+};
+
 // The kernels of a factorization follow one another on one stream, and the
 // small ones take a few microseconds each, about as long as the stream needs
 // to drain one grid and start the next. They are launched with launch_chained,
@@ -72,7 +92,7 @@ inline bool chain_early(int64_t ctas) {
 
 // Launches kern (as a cluster where that has more than one CTA).
 template <typename... P, typename... Args>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, dim3 cluster, bool early,
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, Lane s, dim3 cluster, bool early,
                            Args... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
@@ -81,7 +101,7 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
   cfg.stream = s;
   cudaLaunchAttribute at[2]{};
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  at[0].val.programmaticStreamSerializationAllowed = early && !s.shared ? 1 : 0;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = cluster.x;
   at[1].val.clusterDim.y = cluster.y;

@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(4 * T) k_gemm_f64(int64_t M, int64_t N, int64_
 
 template <int T, bool TA, bool TB>
 cudaError_t launch_gemm(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
-                        int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, int ks, cudaStream_t s) {
+                        int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, int ks, Lane s) {
   const dim3 grid((unsigned)ceil_div(M, T), (unsigned)ceil_div(N, T), (unsigned)ks);
   cudaError_t e = launch_chained(k_gemm_f64<T, TA, TB>, grid, dim3(4 * T), 0, s, dim3(1, 1, (unsigned)ks),
                                  chain_early((int64_t)grid.x * grid.y * grid.z), M, N, K, alpha, A, lda, B, ldb, beta, C,
@@ -232,7 +232,7 @@ cudaError_t launch_gemm(int64_t M, int64_t N, int64_t K, double alpha, const dou
 
 template <int T>
 cudaError_t launch_gemm_t(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
-                          int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, int ks, cudaStream_t s) {
+                          int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, int ks, Lane s) {
   const bool ta = flags & GEMM_TA, tb = flags & GEMM_TB;
   if (!ta && !tb) return launch_gemm<T, false, false>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, ks, s);
   if (!ta && tb) return launch_gemm<T, false, true>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, ks, s);
@@ -246,7 +246,7 @@ cudaError_t launch_gemm_t(int64_t M, int64_t N, int64_t K, double alpha, const d
 // range over the tiles with work, and no less than one CTA's longest range;
 // each CTA also costs about 120 slots to fill and drain (1 us), a cluster's
 // sum 60 more. Ties go to the larger tile and the smaller split.
-void gemm_shape(int64_t M, int64_t N, int64_t K, unsigned flags, int sms, int* T, int* ks) {
+void gemm_shape(int64_t M, int64_t N, int64_t K, unsigned flags, int sms, int max_split, int* T, int* ks) {
   double best = 0.0;
   const bool tri_k = flags & (GEMM_A_LOWER | GEMM_A_UPPER | GEMM_B_LOWER | GEMM_B_UPPER);
   const bool tri_c = flags & (GEMM_C_LOWER | GEMM_C_UPPER);
@@ -254,7 +254,7 @@ void gemm_shape(int64_t M, int64_t N, int64_t K, unsigned flags, int sms, int* T
     const double gx = (double)ceil_div(M, t), gy = (double)ceil_div(N, t);
     const double tiles = tri_c ? std::max(1.0, 0.5 * gx * gy + 0.5 * std::min(gx, gy)) : gx * gy;
     const double kmean = tri_k ? std::min((double)K, 0.5 * (double)K + 0.5 * t) : (double)K;
-    for (int z = 1; z <= 8; z *= 2) {
+    for (int z = 1; z <= max_split; z *= 2) {
       if (z > 1 && K < BK * z) break;
       const double cta = t * t / 32.0 / z;
       const double fixed = 120.0 + (z > 1 ? 60.0 : 0.0);
@@ -272,12 +272,12 @@ void gemm_shape(int64_t M, int64_t N, int64_t K, unsigned flags, int sms, int* T
 }  // namespace
 
 cudaError_t gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda, const double* B,
-                     int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, cudaStream_t s) {
+                     int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags, Lane s) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   int sms = 148, dev = 0, T = 64, ks = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  gemm_shape(M, N, K, flags, sms, &T, &ks);
+  gemm_shape(M, N, K, flags, sms, s.shared ? 1 : 8, &T, &ks);
   if (ceil_div(N, T) > 65535) return cudaErrorInvalidValue;
   return T == 64 ? launch_gemm_t<64>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, ks, s)
                  : launch_gemm_t<32>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc, flags, ks, s);
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(TRMM_PARTS * TRMM_SMALL_MAX)
 }
 
 cudaError_t trmm_upper_small(int n, const double* A, int64_t lda, bool a_trans, const double* B, int64_t ldb,
-                             double* C, int64_t ldc, cudaStream_t s) {
+                             double* C, int64_t ldc, Lane s) {
   if (n < 1 || n > TRMM_SMALL_MAX) return cudaErrorInvalidValue;
   const int threads = (TRMM_PARTS * n + 31) / 32 * 32;
   cudaError_t e = launch_chained(k_trmm_upper_small, dim3((unsigned)n), dim3((unsigned)threads), 0, s, dim3(1), true,

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(32 * GRAM_RC) k_gram_reduce(const double* part
 
 template <int MAXS>
 cudaError_t launch_diag(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,
-                        cudaStream_t s) {
+                        Lane s) {
   const size_t sm = (size_t)2 * KC * (n | 1) * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(k_gram_diag<MAXS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)(2 * KC * 129 * sizeof(double)));
@@ -237,7 +237,7 @@ cudaError_t launch_diag(const double* A, int64_t lda, int64_t m, int n, const Gr
 
 }  // namespace
 
-GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, int row_unit) {
+GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, int row_unit, bool shared) {
   GramGeom g;
   g.ntile = (int)ceil_div(n, 128);
   g.T = (int)ceil_div(ceil_div(n, g.ntile), 16) * 16;
@@ -258,9 +258,12 @@ GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, in
   const int resident = slots <= 8 ? 3 : (slots <= 16 ? 2 : 1);
   const double clocks = (double)m * n * (n + 1) / 2 / (2.0 * sms);
   const int64_t per_sm = std::min<int64_t>(std::max(1, ctas_per_sm), clocks >= 35000.0 * resident ? resident : 1);
-  // as many ranges as fit in that many whole waves, none shorter than 8 rows
+  // as many ranges as fit in that many whole waves, none shorter than 8 rows;
+  // on a shared lane more and shorter ones, none shorter than 32 rows
   int64_t want = std::max<int64_t>(1, per_sm * sms / items);
   want = std::min<int64_t>(want, std::max<int64_t>(1, m / 8));
+  if (shared)
+    want = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, ctas_per_sm) * sms / items, m / 32));
   if (max_splits > 0) want = std::min<int64_t>(want, max_splits);
   g.rows_per_split = ceil_div(ceil_div(m, want), row_unit) * row_unit;
   g.nsplit = std::max<int64_t>(1, ceil_div(m, g.rows_per_split));
@@ -268,7 +271,7 @@ GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, in
 }
 
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,
-                          cudaStream_t s) {
+                          Lane s) {
   if (g.ntile == 1) {
     const int slots = gram_slots(n);
     if (slots <= 8) return launch_diag<8>(A, lda, m, n, g, partial, s);
@@ -286,7 +289,7 @@ cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const 
   return cudaGetLastError();
 }
 
-cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw, cudaStream_t s) {
+cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw, Lane s) {
   dim3 block(32 * GRAM_RC);
   dim3 grid((unsigned)ceil_div(n, 32), (unsigned)n);
   cudaError_t e = launch_chained(k_gram_reduce, grid, block, 0, s, dim3(1), true, partial, g.nsplit, g.T, g.ntile,

@@ -29,12 +29,13 @@ struct GramGeom {
   size_t partial_doubles() const { return (size_t)nsplit * ntiles_total * T * T; }
 };
 // ctas_per_sm: most Gram CTAs per SM (an autotuned knob); row_unit: the ranges'
-// row counts are multiples of it.
-GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm = 4, int row_unit = 4);
+// row counts are multiples of it; shared: for a shared lane (that
+// many waves of CTAs).
+GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm = 4, int row_unit = 4, bool shared = false);
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g,
-                          double* partial, cudaStream_t s);
+                          double* partial, Lane s);
 cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw,
-                        cudaStream_t s);
+                        Lane s);
 
 // ---------------------------------------------------------------- Q-form
 // Q = A Rinv for upper-triangular Rinv (Algorithm CQR step 3).
@@ -45,17 +46,17 @@ constexpr int RP_GROUPS = 16;  // column groups of the packed R^-1 (the Q-form's
 size_t rpack_doubles(int n);
 // Rp[g][k][c] = Rinv(k, j) for k <= j = g*w + c - lead, else 0, with lead =
 // w ceil(n/w) - n (c < w rounded up to even); Rinv = Y^T.
-cudaError_t pack_rinv_from_lower(const double* Y, int64_t ldy, int n, double* Rp, cudaStream_t s);
+cudaError_t pack_rinv_from_lower(const double* Y, int64_t ldy, int n, double* Rp, Lane s);
 // Same from an upper-triangular Rinv (strictly lower part ignored).
-cudaError_t pack_rinv_from_upper(const double* Rinv, int64_t ld, int n, double* Rp, cudaStream_t s);
+cudaError_t pack_rinv_from_upper(const double* Rinv, int64_t ld, int n, double* Rp, Lane s);
 // Q may alias A (each CTA reads its whole row panel before writing it).
 cudaError_t qform_small(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q,
-                        int64_t ldq, cudaStream_t s);
+                        int64_t ldq, Lane s);
 // Fused: Q = A Rinv and the partial Grams of Q (same layout as gram_partials
 // with geometry g, which must have T >= n, i.e. one diagonal tile).
 bool qform_gram_fusable(int n);
 cudaError_t qform_gram_small(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q,
-                             int64_t ldq, const GramGeom& g, double* partial, cudaStream_t s);
+                             int64_t ldq, const GramGeom& g, double* partial, Lane s);
 
 // ---------------------------------------------------------------- GEMM
 // C = alpha op(A) op(B) + beta C, FP64, column-major. Structure flags let
@@ -75,13 +76,13 @@ enum : unsigned {
 // per tile, whose partial sums are added in a fixed order (deterministic).
 cudaError_t gemm_f64(int64_t M, int64_t N, int64_t K, double alpha, const double* A, int64_t lda,
                      const double* B, int64_t ldb, double beta, double* C, int64_t ldc, unsigned flags,
-                     cudaStream_t s);
+                     Lane s);
 
 // R = op(A) B for upper-triangular n x n factors, n <= TRMM_SMALL_MAX, one
 // launch; op(A) = A^T (A lower) when a_trans. C below the diagonal is zeroed.
 constexpr int TRMM_SMALL_MAX = 128;
 cudaError_t trmm_upper_small(int n, const double* A, int64_t lda, bool a_trans, const double* B, int64_t ldb,
-                             double* C, int64_t ldc, cudaStream_t s);
+                             double* C, int64_t ldc, Lane s);
 
 // ---------------------------------------------------------------- CholInv
 // [L, Y] = CholInv(W) (Algorithm 1): recursive halving with FP64 GEMMs and
@@ -95,32 +96,32 @@ constexpr int CHOLINV_LEAF = 128;  // largest leaf
 // may share storage with an output.
 cudaError_t cholinv_leaf(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                          double* Rt, int64_t ldrt, double* Rp, int rpw, DevStatus* st, int pass, long long off,
-                         cudaStream_t s);
+                         Lane s);
 // With Rt, also R = L^T (ld ldrt, zeros below the diagonal); with Rp, also
 // the Q-form's packed R^-1 (pack_rinv_from_lower). A leaf's kernel writes
 // everything; otherwise the transpose and the packing are launches of their own.
 cudaError_t cholinv(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
-                    double* work, double* U, DevStatus* st, int pass, cudaStream_t s, double* Rt = nullptr, int64_t ldrt = 0, double* Rp = nullptr);
+                    double* work, double* U, DevStatus* st, int pass, Lane s, double* Rt = nullptr, int64_t ldrt = 0, double* Rp = nullptr);
 // Inverse depth (the paper's triangular inverted blocks): the top `depth`
 // halvings form L21 = W21 L11^-T by block forward substitution and leave Y21
 // zero, so Y holds the inverses of L's diagonal blocks only. T is scratch of
 // n x right_solve_temp_cols(n) doubles (ld ldt >= n).
 cudaError_t cholinv_depth(int n, const double* W, int64_t ldw, double* L, int64_t ldl, double* Y, int64_t ldy,
                           double* work, double* U, double* T, int64_t ldt, DevStatus* st, int pass, int depth,
-                          cudaStream_t s);
+                          Lane s);
 // X = B L^-T (M x N) for lower-triangular L whose diagonal-block inverses of a
 // depth-`depth` halving are in Y: X1 = B1 L11^-T, X2 = (B2 - X1 L21^T) L22^-T.
 // X may equal B. T is scratch of M x right_solve_temp_cols(N) (ld ldt >= M).
 cudaError_t right_solve(int64_t M, int N, const double* B, int64_t ldb, double* X, int64_t ldx, const double* L,
                         int64_t ldl, const double* Y, int64_t ldy, int depth, double* T, int64_t ldt,
-                        cudaStream_t s);
+                        Lane s);
 int right_solve_temp_cols(int n);
 // Shifted CholeskyQR: W += s I, s = 11 (m n + n (n+1)) 2^-53 trace(W).
 cudaError_t add_shift(double* W, int64_t ldw, int n, int64_t m, cudaStream_t s);
 // R = L^T (upper) with zeros below the diagonal.
-cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int64_t ldr, cudaStream_t s);
+cudaError_t transpose_lower(const double* L, int64_t ldl, int n, double* R, int64_t ldr, Lane s);
 // R = upper part of X with zeros below the diagonal.
-cudaError_t copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr, cudaStream_t s);
+cudaError_t copy_upper(const double* X, int64_t ldx, int n, double* R, int64_t ldr, Lane s);
 
 // ---------------------------------------------------------------- Ozaki
 // Split-precision Gram and Q-form on BF16 tensor cores (see ozaki.cu).
@@ -212,8 +213,8 @@ cudaError_t status_merge(DevStatus* outer, const DevStatus* inner, int64_t col0,
 // c = Q^T b as split-m partials, then x solves R x = c (back substitution).
 int64_t gemv_splits(int64_t m, int n);
 cudaError_t gemv_t_partials(const double* Q, int64_t ldq, int64_t m, int n, const double* b, int64_t nsplit,
-                            double* partial, cudaStream_t s);
+                            double* partial, Lane s);
 cudaError_t lstsq_solve(const double* partial, int64_t nsplit, int n, const double* R, int64_t ldr, double* x,
-                        cudaStream_t s);
+                        Lane s);
 
 }  // namespace cqr2

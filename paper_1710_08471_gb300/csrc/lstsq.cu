@@ -225,7 +225,7 @@ int64_t gemv_splits(int64_t m, int n) {
 }
 
 cudaError_t gemv_t_partials(const double* Q, int64_t ldq, int64_t m, int n, const double* b, int64_t nsplit,
-                            double* partial, cudaStream_t s) {
+                            double* partial, Lane s) {
   const int gpc = gemv_groups(n);
   const int64_t rows_per = ceil_div(ceil_div(m, nsplit), 32) * 32;  // ranges start on 256-byte lines
   dim3 grid((unsigned)(nsplit / (GW / gpc)), (unsigned)ceil_div(n, gpc * GC));
@@ -237,7 +237,7 @@ cudaError_t gemv_t_partials(const double* Q, int64_t ldq, int64_t m, int n, cons
 }
 
 cudaError_t lstsq_solve(const double* partial, int64_t nsplit, int n, const double* R, int64_t ldr, double* x,
-                        cudaStream_t s) {
+                        Lane s) {
   const size_t sm = ((size_t)n + (solve_width(n) < ST ? ST : 0)) * sizeof(double);
   if (sm > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_lstsq_solve, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);

@@ -192,7 +192,7 @@ static_assert(QFORM_ALONE_SMEM >= 256 * PANEL * (int)sizeof(double), "the widest
 
 template <int W>
 cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q, int64_t ldq,
-                         cudaStream_t s) {
+                         Lane s) {
   const size_t sm = (size_t)n * PANEL * sizeof(double);
   auto kern = k_qform_small<W>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, QFORM_ALONE_SMEM);
@@ -200,8 +200,9 @@ cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const d
   const int64_t npanels = ceil_div(m, PANEL);
   int per_sm = 1;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, QT, sm);
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(npanels, (int64_t)sm_count() * std::max(1, per_sm)));
-  const bool early = chain_early(2 * grid);
+  const int64_t waves = s.shared ? 4 : 1;
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(npanels, waves * sm_count() * std::max(1, per_sm)));
+  const bool early = chain_early(2 * grid) && !s.shared;
   e = launch_chained(kern, dim3((unsigned)grid), dim3(QT), early ? (size_t)QFORM_ALONE_SMEM : sm, s, dim3(1), early, A,
                      lda, m, n, Rp, Q, ldq, npanels);
   if (e != cudaSuccess) return e;
@@ -211,7 +212,7 @@ cudaError_t launch_qform(const double* A, int64_t lda, int64_t m, int n, const d
 
 template <int W, int MAXS>
 cudaError_t launch_fused(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q, int64_t ldq,
-                         const GramGeom& g, double* partial, cudaStream_t s) {
+                         const GramGeom& g, double* partial, Lane s) {
   static_assert(MAXS >= gram_slots(16 * W > 128 ? 128 : 16 * W), "slots of the widest matrix of this group width");
   const size_t sm = ((size_t)n * PANEL + (size_t)PANEL * (n | 1)) * sizeof(double);
   auto kern = k_qform_gram_small<W, MAXS>;
@@ -234,7 +235,7 @@ size_t rpack_doubles(int n) {
   return (size_t)NGROUP * n * (w ? pitch_of(w) : 0);
 }
 
-static cudaError_t pack(const double* X, int64_t ldx, int n, bool lower, double* Rp, cudaStream_t s) {
+static cudaError_t pack(const double* X, int64_t ldx, int n, bool lower, double* Rp, Lane s) {
   const int w = qform_group_width(n);
   if (!w) return cudaErrorInvalidValue;
   const int64_t total = (int64_t)rpack_doubles(n);
@@ -246,16 +247,16 @@ static cudaError_t pack(const double* X, int64_t ldx, int n, bool lower, double*
   return cudaGetLastError();
 }
 
-cudaError_t pack_rinv_from_lower(const double* Y, int64_t ldy, int n, double* Rp, cudaStream_t s) {
+cudaError_t pack_rinv_from_lower(const double* Y, int64_t ldy, int n, double* Rp, Lane s) {
   return pack(Y, ldy, n, true, Rp, s);
 }
 
-cudaError_t pack_rinv_from_upper(const double* Rinv, int64_t ld, int n, double* Rp, cudaStream_t s) {
+cudaError_t pack_rinv_from_upper(const double* Rinv, int64_t ld, int n, double* Rp, Lane s) {
   return pack(Rinv, ld, n, false, Rp, s);
 }
 
 cudaError_t qform_small(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q, int64_t ldq,
-                        cudaStream_t s) {
+                        Lane s) {
   switch (qform_group_width(n)) {
     case 1: return launch_qform<1>(A, lda, m, n, Rp, Q, ldq, s);
     case 2: return launch_qform<2>(A, lda, m, n, Rp, Q, ldq, s);
@@ -280,7 +281,7 @@ cudaError_t qform_small(const double* A, int64_t lda, int64_t m, int n, const do
 bool qform_gram_fusable(int n) { return n >= 1 && n <= 128; }
 
 cudaError_t qform_gram_small(const double* A, int64_t lda, int64_t m, int n, const double* Rp, double* Q,
-                             int64_t ldq, const GramGeom& g, double* partial, cudaStream_t s) {
+                             int64_t ldq, const GramGeom& g, double* partial, Lane s) {
   if (!qform_gram_fusable(n) || g.ntile != 1 || g.T < n) return cudaErrorInvalidValue;
   switch (qform_group_width(n)) {
     case 1: return launch_fused<1, 8>(A, lda, m, n, Rp, Q, ldq, g, partial, s);

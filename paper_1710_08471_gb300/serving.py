@@ -100,6 +100,12 @@ class CudaExecutor:
         if p is None:
             prec = self.precision if n <= 1024 else cq.CQR2_FP64
             p = cq.Plan(self.m_max, n, precision=prec, stream=self.streams[slot])
+            if prec == cq.CQR2_FP64:
+                # The other slots' requests run beside this one's. On a server of one
+                # slot too, so that a result does not depend on the slots. Split
+                # precision gained too little (1697 -> 1718 requests/s) to slow its
+                # one-slot server.
+                p.set_shared(True)
             self.plans[slot][n] = p
             self.workspace_bytes += p.workspace_bytes
         return p
