@@ -141,6 +141,14 @@ cudaError_t copy_cols(double* dst, int64_t ldd, const double* src, int64_t lds, 
                            kind, s);
 }
 
+// A captured launch sequence no longer applies.
+void drop_graph(cqr2_plan_st* p) {
+  if (p->gexec) cudaGraphExecDestroy(p->gexec);
+  if (p->graph) cudaGraphDestroy(p->graph);
+  p->gexec = nullptr;
+  p->graph = nullptr;
+}
+
 cqr2_status_t check_device(const cqr2_plan_st* p) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return CQR2_ERR_CUDA;
@@ -742,6 +750,7 @@ cqr2_status_t cqr2_plan_set_panel_width(cqr2_plan_t p, int64_t b) {
   if (b >= p->n) b = 0;  // one panel is plain CholeskyQR2
   if (b == p->panel_b) return CQR2_OK;
   if (cudaStreamSynchronize(p->stream) != cudaSuccess) return CQR2_ERR_CUDA;
+  drop_graph(p);  // its nodes use the panels' workspaces
   cqr2_plan_destroy(p->pan_full);
   cqr2_plan_destroy(p->pan_tail);
   cudaFree(p->pan_C);
@@ -766,8 +775,7 @@ cqr2_status_t cqr2_plan_set_panel_width(cqr2_plan_t p, int64_t b) {
     return r;
   }
   p->panel_b = b;
-  // the panels' plans too; a captured graph of the unpaneled sequence goes
-  return cqr2_plan_set_shared(p, p->shared);
+  return cqr2_plan_set_shared(p, p->shared);  // and its panels' plans
 }
 
 cqr2_status_t cqr2_plan_split_slices(cqr2_plan_t plan, int32_t* slices) {
@@ -799,10 +807,7 @@ cqr2_status_t cqr2_factor_rows(cqr2_plan_t p, int64_t m, const double* dA, int64
     const bool same = p->gexec && p->gkey.A == dA && p->gkey.Q == dQ && p->gkey.R == dR && p->gkey.lda == lda &&
                       p->gkey.ldq == ldq && p->gkey.ldr == ldr && p->gkey.m == m;
     if (!same) {
-      if (p->gexec) cudaGraphExecDestroy(p->gexec);
-      if (p->graph) cudaGraphDestroy(p->graph);
-      p->gexec = nullptr;
-      p->graph = nullptr;
+      drop_graph(p);
       TRY(cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal));
       const int64_t l0 = launch_count();
       r = factor_any(p, dA, lda, dQ, ldq, dR, ldr);
@@ -840,10 +845,7 @@ cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t p, int32_t ctas_per_sm) {
   if (!p || ctas_per_sm < 1 || ctas_per_sm > GRAM_CPS_MAX) return CQR2_ERR_INVALID_ARG;
   p->gram_cps = ctas_per_sm;
   p->cm = 0;  // recompute the geometry on the next call
-  if (p->gexec) cudaGraphExecDestroy(p->gexec);
-  if (p->graph) cudaGraphDestroy(p->graph);
-  p->gexec = nullptr;
-  p->graph = nullptr;
+  drop_graph(p);
   return CQR2_OK;
 }
 
@@ -853,10 +855,7 @@ cqr2_status_t cqr2_plan_set_shared(cqr2_plan_t p, int32_t shared) {
   p->cm = 0;  // recompute the geometry on the next call
   if (p->pan_full) cqr2_plan_set_shared(p->pan_full, shared);
   if (p->pan_tail) cqr2_plan_set_shared(p->pan_tail, shared);
-  if (p->gexec) cudaGraphExecDestroy(p->gexec);
-  if (p->graph) cudaGraphDestroy(p->graph);
-  p->gexec = nullptr;
-  p->graph = nullptr;
+  drop_graph(p);
   return CQR2_OK;
 }
 
@@ -873,10 +872,7 @@ cqr2_status_t cqr2_plan_set_inverse_depth(cqr2_plan_t p, int32_t depth) {
     p->ldt = ldt;
   }
   p->inv_depth = depth;
-  if (p->gexec) cudaGraphExecDestroy(p->gexec);  // a captured launch sequence no longer applies
-  if (p->graph) cudaGraphDestroy(p->graph);
-  p->gexec = nullptr;
-  p->graph = nullptr;
+  drop_graph(p);
   return CQR2_OK;
 }
 
@@ -903,10 +899,7 @@ cqr2_status_t cqr2_selftest_wait_timeout(int64_t polls, void* stream) {
 cqr2_status_t cqr2_plan_set_fused(cqr2_plan_t p, int32_t fused) {
   if (!p) return CQR2_ERR_INVALID_ARG;
   p->fused = fused && !p->oz_S && qform_gram_fusable((int)p->n) && p->small;
-  if (p->gexec) cudaGraphExecDestroy(p->gexec);
-  if (p->graph) cudaGraphDestroy(p->graph);
-  p->gexec = nullptr;
-  p->graph = nullptr;
+  drop_graph(p);
   return CQR2_OK;
 }
 
