@@ -165,41 +165,20 @@ static __device__ __noinline__ double oz_xy_to_double_cold(long long X, long lon
 #define OZ_XY_COLD oz_xy_to_double
 #endif
 
-// Faster conversion of T = X 2^24 + Y (|X| < 2^61, |Y| < 2^55) to within one
-// ulp of T 2^E: scale T by 2^-sh so that it fits 62 bits (the bits of Y that
-// fall off are below 2^-61 of it), then round that int64 to nearest.
-OZ_HD double oz_xy_to_double_fast(long long X, long long Y, int E) {
-  const unsigned long long ax = X < 0 ? 0ull - (unsigned long long)X : (unsigned long long)X;
-  const int bl = 64 - oz_clz64(ax);  // bit length of |X|
-  const int sh = bl > 38 ? bl - 38 : 0;
-  const long long Z = (long long)((unsigned long long)X << (24 - sh)) + (Y >> sh);
-  const bool neg = Z < 0;
-  unsigned long long u = neg ? 0ull - (unsigned long long)Z : (unsigned long long)Z;
-  if (u == 0) return 0.0;
-  const int lz = oz_clz64(u);
-  u <<= lz;
-  unsigned long long mant = u >> 11;
-  const unsigned long long rb = (u >> 10) & 1ull, st = (u & 0x3FFull) != 0 ? 1ull : 0ull;
-  const int biased = 63 - lz + E + sh + 1023;
-  if (biased < 1) return OZ_XY_COLD(X, Y, E);  // subnormal: rare, exact path
-  mant += rb & (st | (mant & 1ull));
-  unsigned long long bits = ((unsigned long long)(biased - 1) << 52) + mant;
-  if (biased > 2046) bits = 0x7FF0000000000000ull;
-  return oz_bits_to_double(bits | (neg ? 1ull << 63 : 0ull));
-}
-
-// The same for a group of outputs with one shift: T 2^-(24-s) = X 2^s + Y
-// 2^-(24-s) fits 62 bits for every output of the group when s = min(24, 62 -
-// (bits of the largest |X|)), and what falls off Y (rounded) is then below
-// 2^-61 of the group's largest |T|. The hardware converts that integer with one
-// correct rounding (one FP64 operation), and the exponent is added to its bits:
-// about a quarter of the instructions of the normalising sequence above, which
-// was most of the Q-form's epilogue.
-// h: the OR over the group of oz_high_bits(X).
+// Faster conversion of T = X 2^24 + Y (|X| < 2^61, |Y| < 2^55) to within one ulp
+// of T 2^E: T 2^-(24-s) = X 2^s + Y 2^-(24-s) fits 62 bits when s = min(24, 62 -
+// (bits of |X|)), and what falls off Y is then below 2^-61 of |T|. The hardware
+// converts that integer with one correct rounding (one FP64 operation), and the
+// exponent is added to its bits. Each output has its own shift: with one for a
+// group of outputs the bits that fall off would be below 2^-61 of the group's
+// largest only, and it was no faster (group shift of a thread's four or eight
+// outputs with 64-bit shifts, and this: 2^23 x 128 29.13, 29.15 ms; 2^21 x 512
+// 57.7, 57.1; 1000037 x 200 with six slices 7.63, 7.70).
 OZ_HD unsigned oz_high_bits(long long X) {
   const int hi = (int)(X >> 32);
   return (unsigned)(hi ^ (hi >> 31));
 }
+// h: oz_high_bits(X), or their OR over outputs that share a shift.
 OZ_HD int oz_group_shift(unsigned h) {
 #if defined(__CUDA_ARCH__)
   const int lz = __clz((int)h);
@@ -208,29 +187,51 @@ OZ_HD int oz_group_shift(unsigned h) {
 #endif
   return lz - 2 < 24 ? lz - 2 : 24;
 }
-// The conversion without its rare cases, so that a kernel can run several side
-// by side without branches; ok is false for zero and for a result outside the
-// normal range, which oz_xy_to_double_group (below) then forms.
-OZ_HD double oz_xy_to_double_group_fast(long long X, long long Y, int s, int E, bool* ok) {
-  const int sh = 24 - s;
-  const long long Z = (long long)((unsigned long long)X << s) + ((Y + ((1ll << sh) >> 1)) >> sh);
+OZ_HD unsigned oz_funnel_l(unsigned lo, unsigned hi, int s) {  // high word of (hi:lo) << s, s < 32
+#if defined(__CUDA_ARCH__)
+  return __funnelshift_l(lo, hi, s);
+#else
+  return (unsigned)(((((unsigned long long)hi << 32) | lo) << s) >> 32);
+#endif
+}
+// floor(X 2^s + Y 2^-(24-s)): T = hi 2^24 + lo with lo's 24 bits in one word, so
+// that two funnel shifts form it (64-bit shifts by a variable count take several
+// instructions each).
+OZ_HD long long oz_shifted_int(long long X, long long Y, int s) {
+  const unsigned long long hi = (unsigned long long)(X + (Y >> 24));
+  const unsigned h1 = (unsigned)(hi >> 32), h0 = (unsigned)hi, lo = (unsigned)Y << 8;
+  return (long long)(((unsigned long long)oz_funnel_l(h0, h1, s) << 32) | oz_funnel_l(lo, h0, s));
+}
+// Z 2^e without the rare cases, so that a kernel can run several side by side
+// without branches; ok is false for zero and for a result outside the normal range.
+OZ_HD double oz_int_to_double(long long Z, int e, bool* ok) {
 #if defined(__CUDA_ARCH__)
   const double d = __ll2double_rn(Z);
 #else
   const double d = (double)Z;
 #endif
   const unsigned long long b = (unsigned long long)oz_double_bits(d);
-  const int e = E + sh, ex = (int)((b >> 52) & 0x7FF);
+  const int ex = (int)((b >> 52) & 0x7FF);
   *ok = ex != 0 && (unsigned)(ex + e - 1) < 2046u;
   return oz_bits_to_double(b + ((unsigned long long)(long long)e << 52));
 }
+// With a given shift, Y rounded to it; the rare cases exactly.
 OZ_HD double oz_xy_to_double_group(long long X, long long Y, int s, int E) {
+  const long long Z = oz_shifted_int(X, Y + (0x800000u >> s), s);
   bool ok;
-  const double v = oz_xy_to_double_group_fast(X, Y, s, E, &ok);
+  const double v = oz_int_to_double(Z, E + 24 - s, &ok);
   if (ok) return v;
-  const int sh = 24 - s;
-  const long long Z = (long long)((unsigned long long)X << s) + ((Y + ((1ll << sh) >> 1)) >> sh);
   return Z == 0 ? 0.0 : OZ_XY_COLD(X, Y, E);
+}
+// With the output's own shift: without its rare cases, and complete.
+OZ_HD double oz_xy_to_double_fast_normal(long long X, long long Y, int E, bool* ok) {
+  const int s = oz_group_shift(oz_high_bits(X));
+  return oz_int_to_double(oz_shifted_int(X, Y, s), E + 24 - s, ok);
+}
+OZ_HD double oz_xy_to_double_fast(long long X, long long Y, int E) {
+  bool ok;
+  const double v = oz_xy_to_double_fast_normal(X, Y, E, &ok);
+  return ok ? v : oz_xy_to_double_group(X, Y, oz_group_shift(oz_high_bits(X)), E);
 }
 
 }  // namespace cqr2

@@ -22,7 +22,8 @@
 // output (T = X 2^24 + Y, X: groups 0-3, Y: groups 4-6), which stays exact
 // as well. The only roundings are the one of x' and the final conversion to
 // FP64: correctly rounded for the Gram (integer operations), within one ulp for
-// the Q-form (a shorter sequence; far below its truncation error).
+// the Q-form (a shorter sequence, each output to 2^-61 of itself before its one
+// rounding; far below the error of the dropped products).
 //
 // Kernel: persistent, one CTA per SM. BF16 operands in 128-byte swizzled
 // shared memory, loaded by TMA from the column slice planes, stored K-block
@@ -896,10 +897,6 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
         constexpr int CB = CPT == 8 ? 8 : 4;
 #pragma unroll
         for (int cb = 0; cb < CPT; cb += CB) {
-          unsigned h = 0;  // one shift for these outputs of the thread
-#pragma unroll
-          for (int cc = cb; cc < cb + CB; ++cc) h |= oz_high_bits(X[cc]);
-          const int shift = oz_group_shift(h);
           const int64_t col0 = w.j0 + cs * CPT + cb;
           const int ncol = (int)min((int64_t)CB, p.n - col0);  // may be negative
           double v[CB];
@@ -908,7 +905,7 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
           for (int cc = 0; cc < CB; ++cc) {
             const int e2 = NEB > 1 ? eb[cb + cc < NEB ? cb + cc : 0] : (cc < ncol ? p.eB[col0 + cc] : 0);
             bool fine;
-            v[cc] = oz_xy_to_double_group_fast(X[cb + cc], Y[cb + cc], shift, e2 - 14 - 48, &fine);
+            v[cc] = oz_xy_to_double_fast_normal(X[cb + cc], Y[cb + cc], e2 - 14 - 48, &fine);
             if (!fine && cc < ncol) rare |= 1u << cc;
           }
           if (rare != 0) {
@@ -917,7 +914,7 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
               if (rare >> cc & 1) {
                 const int e2 = p.eB[col0 + cc];
                 v[cc] = e2 >= EXP_NONFINITE ? __longlong_as_double(0x7FF8000000000000ll)
-                                            : oz_xy_to_double_group(X[cb + cc], Y[cb + cc], shift, e2 - 14 - 48);
+                                            : oz_xy_to_double_fast(X[cb + cc], Y[cb + cc], e2 - 14 - 48);
               }
           }
           if (row < nrow) {
