@@ -139,6 +139,15 @@ RS_HD void chol_rsqrt_tight(double d, double* r, double* l) {
   *r = fma(0.5 * r0, fma(-lo, r0, fma(-l0, r0, 1.0)), r0);
 }
 
+// a / d, correctly rounded, from r = 1 / d (correctly rounded): the product and
+// one correction by its exact remainder (P. Markstein, IBM J. Res. Dev. 34(1),
+// 1990), for where many quotients share a divisor. For intermediates in the
+// normal range.
+RS_HD double rs_quotient(double a, double d, double r) {
+  const double q = a * r;
+  return fma(fma(-q, d, a), r, q);
+}
+
 // Single-precision seed of 1/f, f in [1, 2).
 RS_HD float rs_rcp_seed(float f) {
 #if defined(__CUDA_ARCH__)

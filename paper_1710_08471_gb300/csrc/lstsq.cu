@@ -3,7 +3,9 @@
 // partial sums (summed in a fixed order) and solves R x = c by back
 // substitution in one CTA.
 #include <algorithm>
+#include <type_traits>
 
+#include "fp64_rsqrt.cuh"
 #include "kernels.h"
 
 namespace cqr2 {
@@ -82,10 +84,14 @@ __global__ void __launch_bounds__(GT) k_gemv_t_partial(const double* Q, int64_t 
 //    fixed order);
 //  - one warp solves the 32 x 32 diagonal block from registers, in the form
 //    c_i -= (R_ik / R_kk) c_k, so that a column's chain is a shuffle and an
-//    FMA, and x = c / R_kk comes last, for all columns at once. Two warps take
+//    FMA, and x = c / R_kk comes last, for all columns at once. The quotients
+//    are correctly rounded, from the diagonal's reciprocals and a correction
+//    each (products with the reciprocals alone: 0.8 us less at 16 columns and
+//    2 us at 32, none at 100 and more, and at 16 columns an error of the solve
+//    9% above that with divisions). Two warps take
 //    the blocks in turn: one loads and scales its next block while the other
-//    solves (where a diagonal entry is too small or too large for its
-//    reciprocal, the block is solved with divisions);
+//    solves (where an entry is too small or too large for this, the block is
+//    solved with divisions);
 //  - the other warps then update the rows above the block, two lanes to a row
 //    with 16 values of R each, loaded ahead of the barrier.
 // n = 256: 356 -> 51 us, n = 100: 90 -> 28 us.
@@ -134,18 +140,36 @@ __global__ void __launch_bounds__(ST) k_lstsq_solve(const double* partial, int64
     double rr[SB];  // this lane's row of the diagonal block, divided by the columns' diagonal entries
     double rinv = 1.0, rd = 1.0;
     bool safe = true;
-    auto load_block = [&](int B0) {
+    auto load_block = [&](int B0) {  // unscaled
 #pragma unroll
       for (int k = 0; k < SB; ++k)
         rr[k] = (lane < k && B0 + k < n) ? R[(B0 + lane) + (int64_t)(B0 + k) * ldr] : 0.0;
       rd = B0 + lane < n ? R[(B0 + lane) + (int64_t)(B0 + lane) * ldr] : 1.0;
       rinv = 1.0 / rd;
       const double a = fabs(rd);
-      safe = __all_sync(0xffffffffu, a > 0x1p-500 && a < 0x1p500);
+      int top = 0;  // high word of the largest entry
 #pragma unroll
-      for (int k = 0; k < SB; ++k) rr[k] *= __shfl_sync(0xffffffffu, rinv, k);
+      for (int k = 0; k < SB; ++k) top = max(top, __double2hiint(rr[k]) & 0x7FFFFFFF);
+      safe = __all_sync(0xffffffffu, a > 0x1p-500 && a < 0x1p500 && top < (1023 + 500) << 20);
     };
-    if (last - warp >= 0) load_block((last - warp) * SB);
+    // A block's 93 operations for the quotients take 3 us: in three parts, they
+    // hide behind an update, the other warp's solve and the update after that
+    // (8192 x 256: 2575 us with products, 2593 in one part, 2584 in three).
+    constexpr int K1 = 11, K2 = 21;
+    auto scale = [&](int B0, auto from, auto to) {
+#pragma unroll
+      for (int k = decltype(from)::value; k < decltype(to)::value; ++k)
+        if (B0 + k < n) rr[k] = rs_quotient(rr[k], __shfl_sync(0xffffffffu, rd, k), __shfl_sync(0xffffffffu, rinv, k));
+    };
+    using std::integral_constant;
+    const integral_constant<int, 1> k0{};
+    const integral_constant<int, K1> k1{};
+    const integral_constant<int, K2> k2{};
+    const integral_constant<int, SB> k3{};
+    if (last - warp >= 0) {
+      load_block((last - warp) * SB);
+      scale((last - warp) * SB, k0, k3);
+    }
     for (int blk = last; blk >= 0; --blk) {
       const int B0 = blk * SB;
       const bool mine = ((last - blk) & 1) == warp;
@@ -154,7 +178,8 @@ __global__ void __launch_bounds__(ST) k_lstsq_solve(const double* partial, int64
         if (safe) {
 #pragma unroll
           for (int k = SB - 1; k >= 1; --k) ci = fma(-rr[k], __shfl_sync(0xffffffffu, ci, k), ci);
-          ci *= rinv;
+          const double q = rs_quotient(ci, rd, rinv);
+          ci = isfinite(q) ? q : ci * rinv;
         } else {
 #pragma unroll 1
           for (int k = min(SB, n - B0) - 1; k >= 0; --k) {
@@ -167,9 +192,18 @@ __global__ void __launch_bounds__(ST) k_lstsq_solve(const double* partial, int64
           c[B0 + lane] = ci;
           x[B0 + lane] = ci;
         }
+      } else if (blk >= 1 && blk < last) {
+        scale(B0 - SB, k1, k2);
       }
       __syncthreads();
-      if (mine && blk >= 2) load_block(B0 - 2 * SB);
+      if (mine) {
+        if (blk >= 2) {
+          load_block(B0 - 2 * SB);
+          scale(B0 - 2 * SB, k0, k1);
+        }
+      } else if (blk >= 1 && blk < last) {
+        scale(B0 - SB, k2, k3);
+      }
       __syncthreads();
     }
   } else {
