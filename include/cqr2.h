@@ -163,9 +163,10 @@ cqr2_status_t cqr2_lstsq_rows(cqr2_plan_t plan, int64_t m, const double* dA, int
                               double* dx, double* dQ, int64_t ldq, double* dR, int64_t ldr, cqr2_info_t* info);
 
 /* Tuning knobs of a plan (set by the autotuner, cqr2_autotune, or by hand):
- * the largest number of Gram CTAs per SM (1..8, default 4; the library uses
- * fewer where more would not help), and whether to fuse the
- * pass-1 Q-form with the pass-2 Gram (honoured only where CQR2_FUSED is). */
+ * the largest number of Gram CTAs per SM (1..8, default 4; an FP64 Gram uses at
+ * most 3 up to 63 columns, 2 up to 90 and 1 beyond, a shared plan at most 4, and
+ * a split-precision Gram none of this), and whether to fuse the pass-1 Q-form
+ * with the pass-2 Gram (honoured only where CQR2_FUSED is). */
 cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t plan, int32_t ctas_per_sm);
 cqr2_status_t cqr2_plan_set_fused(cqr2_plan_t plan, int32_t fused);
 
@@ -173,7 +174,8 @@ cqr2_status_t cqr2_plan_set_fused(cqr2_plan_t plan, int32_t fused);
  * default, or 1). Launch shapes are otherwise chosen for a call that has the
  * GPU to itself; with 1 they let the streams' kernels interleave, which lowers
  * the latency of many calls at a time and slows one alone (the smallest most). The result
- * is the same up to rounding. Not for use while the plan's stream has a call in
+ * is the same up to rounding. The first 1 allocates room for more partial Grams
+ * (CQR2_ERR_OOM if that fails). Not for use while the plan's stream has a call in
  * flight. */
 cqr2_status_t cqr2_plan_set_shared(cqr2_plan_t plan, int32_t shared);
 
@@ -336,7 +338,7 @@ typedef struct {
   int32_t gram_ctas;   /* best Gram CTAs per SM */
   int32_t fused;       /* best fusion choice */
   double ms;           /* its time per factorization */
-  int32_t candidates;  /* configurations timed */
+  int32_t candidates;  /* configurations compared (those with the same launches are timed once) */
 } cqr2_tune_result_t;
 
 /* Time the candidate configurations (Gram CTAs per SM 1, 2, 4, 8; fused or

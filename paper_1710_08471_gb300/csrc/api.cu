@@ -71,6 +71,7 @@ struct cqr2_plan_st {
   // in row blocks on a copy stream while the pass-1 Gram consumes them, and
   // Q leaves block by block as the last Q-form writes it.
   cudaStream_t copy_stream = nullptr;
+  double* shared_partial = nullptr;  // partials of a shared plan (cqr2_plan_set_shared), if larger
   double* hx_partial = nullptr;  // Gram partials of the row blocks (HX_BLOCKS x hx_cap ranges)
   int64_t hx_cap = 0;
   std::vector<cudaEvent_t> hx_ev;  // [0, HX_BLOCKS): A block in; [HX_BLOCKS, 2 HX_BLOCKS): Q block out; 2 more
@@ -368,7 +369,7 @@ cqr2_status_t factor_impl(cqr2_plan_st* p, const double* dA, int64_t lda, double
         const int64_t r0 = hx_row(p->cm, b), r1 = hx_row(p->cm, b + 1);
         TRY(cudaStreamWaitEvent(s, p->hx_ev[b], 0));
         if (r1 <= r0) continue;
-        const GramGeom gr = gram_geometry(r1 - r0, n, p->hx_cap, p->gram_cps, 4, p->shared);
+        const GramGeom gr = gram_geometry(r1 - r0, n, p->hx_cap, p->gram_cps);
         TRY(gram_partials(dA + r0, lda, r1 - r0, n, gr, p->hx_partial + used * per_split, s));
         used += gr.nsplit;
       }
@@ -592,15 +593,9 @@ cqr2_status_t cqr2_plan_create(cqr2_plan_t* plan, int64_t m, int64_t n, int32_t 
   p->flags = flags;
   p->device = dev;
   p->stream = static_cast<cudaStream_t>(stream);
-  // Size the Gram partials for every row count the plan serves: a smaller m
-  // can round to more (shorter) ranges than m itself, up to the CTA target.
-  p->g = gram_geometry(m, (int)n, 0, GRAM_CPS_MAX);
-  {
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    p->gram_cap = std::max<int64_t>(p->g.nsplit, ceil_div((int64_t)GRAM_CPS_MAX * sms, p->g.ntiles_total));
-    p->g.nsplit = p->gram_cap;
-  }
+  // Gram partials for every row count and knob the plan serves.
+  p->g = gram_geometry(m, (int)n, 0);
+  p->gram_cap = p->g.nsplit = gram_split_capacity((int)n, false);
   p->small = qform_group_width((int)n) > 0;
   p->fused = (flags & CQR2_FUSED) && qform_gram_fusable((int)n);
   p->gemv_nsplit = gemv_splits(m, (int)n);
@@ -621,7 +616,7 @@ cqr2_status_t cqr2_plan_create(cqr2_plan_t* plan, int64_t m, int64_t n, int32_t 
     off[k++] = sz;
     sz += align_up(bytes);
   };
-  take(p->g.partial_doubles() * sizeof(double));                     // 0 partial
+  take(oz_S ? 0 : p->g.partial_doubles() * sizeof(double));         // 0 partial
   take(nn);                                                          // 1 W
   take(nn);                                                          // 2 Wk
   take(nn);                                                          // 3 L
@@ -728,6 +723,7 @@ void cqr2_plan_destroy(cqr2_plan_t plan) {
   }
   for (cudaEvent_t e : plan->hx_ev) cudaEventDestroy(e);
   cudaFree(plan->hx_partial);
+  cudaFree(plan->shared_partial);
   cudaFree(plan->Tsolve);
   cudaFree(plan->hA_dev);
   cudaFree(plan->lsQ);
@@ -851,11 +847,25 @@ cqr2_status_t cqr2_plan_set_gram_ctas(cqr2_plan_t p, int32_t ctas_per_sm) {
 
 cqr2_status_t cqr2_plan_set_shared(cqr2_plan_t p, int32_t shared) {
   if (!p) return CQR2_ERR_INVALID_ARG;
+  const int64_t cap = gram_split_capacity((int)p->n, true);
+  if (shared && !p->oz_S && cap > p->gram_cap) {  // room for the shorter ranges, once
+    const size_t bytes = (size_t)cap * p->g.ntiles_total * p->g.T * p->g.T * sizeof(double);
+    if (cudaMalloc(&p->shared_partial, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      p->shared_partial = nullptr;
+      return CQR2_ERR_OOM;
+    }
+    p->partial = p->shared_partial;
+    p->gram_cap = cap;
+    p->ws_bytes += bytes;
+  }
   p->shared = shared != 0;
   p->cm = 0;  // recompute the geometry on the next call
-  if (p->pan_full) cqr2_plan_set_shared(p->pan_full, shared);
-  if (p->pan_tail) cqr2_plan_set_shared(p->pan_tail, shared);
   drop_graph(p);
+  for (cqr2_plan_st* q : {p->pan_full, p->pan_tail}) {
+    const cqr2_status_t r = q ? cqr2_plan_set_shared(q, shared) : CQR2_OK;
+    if (r != CQR2_OK) return r;
+  }
   return CQR2_OK;
 }
 
@@ -1056,10 +1066,8 @@ cqr2_status_t cqr2_factor_host(cqr2_plan_t p, const double* hA, int64_t lda, dou
   const size_t mn = (size_t)p->m * p->n * sizeof(double);
   if (!p->hA_dev) {
     // Partials for the row-blocked pass-1 Gram: each block may use as many
-    // ranges as the largest CTA target asks for.
-    int sms = 148;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
-    p->hx_cap = std::max<int64_t>(1, ceil_div((int64_t)GRAM_CPS_MAX * sms, p->g.ntiles_total));
+    // ranges as a whole matrix.
+    p->hx_cap = gram_split_capacity((int)p->n, false);
     const size_t part = (size_t)HX_BLOCKS * p->hx_cap * p->g.ntiles_total * p->g.T * p->g.T * sizeof(double);
     if (cudaMalloc(&p->hA_dev, mn) != cudaSuccess || cudaMalloc(&p->hQ_dev, mn) != cudaSuccess ||
         cudaMalloc(&p->hR_dev, (size_t)p->n * p->n * sizeof(double)) != cudaSuccess ||

@@ -413,14 +413,23 @@ cqr2_status_t cqr2_autotune(int64_t m, int64_t n, int32_t precision, cqr2_tune_r
     cudaFree(R);
     return r;
   }
-  const int cps_list[] = {1, 2, 4, 8};
+  const int cps_list[] = {8, 4, 2, 1};
   const int fused_list[] = {0, 1};
   double best = 1e30;
   TuneEntry bestE{4, 1, 0.0};
   int tried = 0;
   for (int f : fused_list) {
     if (f && (precision != CQR2_FP64 || n > 128)) continue;
+    // values that give the same launches are timed once, and the largest stands
+    // for them (it limits nothing at other row counts)
+    int64_t timed[2] = {0, 0};  // rows per range: of the Gram, of the fused kernel
     for (int cps : cps_list) {
+      const int64_t rows[2] = {gram_geometry(m, (int)n, 0, cps).rows_per_split,
+                               gram_geometry(m, (int)n, 0, cps, QFORM_PANEL).rows_per_split};
+      ++tried;
+      const bool same = rows[0] == timed[0] && (!f || rows[1] == timed[1]);
+      if (timed[0] && (same || precision != CQR2_FP64)) continue;
+      std::copy(rows, rows + 2, timed);
       cqr2_plan_set_fused(plan, f);
       cqr2_plan_set_gram_ctas(plan, cps);
       cqr2_factor(plan, A, m, Q, m, R, n, nullptr);  // warm
@@ -432,7 +441,6 @@ cqr2_status_t cqr2_autotune(int64_t m, int64_t n, int32_t precision, cqr2_tune_r
       float ms = 0.f;
       cudaEventElapsedTime(&ms, e0, e1);
       ms /= reps;
-      ++tried;
       if (ms < best) {
         best = ms;
         bestE = TuneEntry{cps, f, ms};

@@ -237,37 +237,53 @@ cudaError_t launch_diag(const double* A, int64_t lda, int64_t m, int n, const Gr
 
 }  // namespace
 
+namespace {
+// CTAs of equal work per row range: one per off-diagonal tile, one per two
+// diagonal tiles.
+int64_t gram_items(int ntile) { return (int64_t)ntile * (ntile - 1) / 2 + ceil_div(ntile, 2); }
+int gram_sms() {
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+// CTAs resident on an SM at a time (few slots per thread).
+int gram_resident(int n) {
+  const int slots = gram_slots(std::min(n, 128));
+  return slots <= 8 ? 3 : (slots <= 16 ? 2 : 1);
+}
+}  // namespace
+
 GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm, int row_unit, bool shared) {
   GramGeom g;
   g.ntile = (int)ceil_div(n, 128);
   g.T = (int)ceil_div(ceil_div(n, g.ntile), 16) * 16;
   g.ntiles_total = g.ntile + g.ntile * (g.ntile - 1) / 2;
-  int dev = 0, sms = 148;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // CTAs of equal work per row range: one per off-diagonal tile, one per two
-  // diagonal tiles.
-  const int64_t items = g.ntiles_total - g.ntile + ceil_div(g.ntile, 2);
-  // CTAs per SM: one, and where several are resident at a time (few slots per
-  // thread) and each still has 35000 clocks (17 us) of FP64 work, that many.
-  // More only cost: filling a CTA's pipeline, writing its partial tiles and
-  // reading them back take 2 to 3 us. Gram and sum together with 1, 2, 3, 4
-  // CTAs per SM: 4096 x 64 29, 32, 41, 41 us; 50021 x 100 435, 451, 463, 474 us;
-  // 131072 x 32 166, 145, 136, 171 us; 262144 x 16 105, 93, 89, 125 us.
-  const int slots = gram_slots((int)std::min<int64_t>(n, 128));
-  const int resident = slots <= 8 ? 3 : (slots <= 16 ? 2 : 1);
+  const int sms = gram_sms();
+  const int64_t items = gram_items(g.ntile);
+  // CTAs per SM: one, and where several are resident at a time and each still
+  // has 35000 clocks (17 us) of FP64 work, that many. More only cost: filling a
+  // CTA's pipeline, writing its partial tiles and reading them back take 2 to
+  // 3 us. Gram and sum together with 1, 2, 3, 4 CTAs per SM: 4096 x 64 29, 32, 41,
+  // 41 us; 50021 x 100 435, 451, 463, 474 us; 131072 x 32 166, 145, 136, 171 us;
+  // 262144 x 16 105, 93, 89, 125 us.
+  const int resident = gram_resident(n), knob = std::max(1, ctas_per_sm);
   const double clocks = (double)m * n * (n + 1) / 2 / (2.0 * sms);
-  const int64_t per_sm = std::min<int64_t>(std::max(1, ctas_per_sm), clocks >= 35000.0 * resident ? resident : 1);
+  const int64_t per_sm = std::min(knob, clocks >= 35000.0 * resident ? resident : 1);
   // as many ranges as fit in that many whole waves, none shorter than 8 rows;
   // on a shared lane more and shorter ones, none shorter than 32 rows
-  int64_t want = std::max<int64_t>(1, per_sm * sms / items);
-  want = std::min<int64_t>(want, std::max<int64_t>(1, m / 8));
-  if (shared)
-    want = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::max(1, ctas_per_sm) * sms / items, m / 32));
+  int64_t want = std::min<int64_t>(per_sm * sms / items, m / 8);
+  if (shared) want = std::min<int64_t>((int64_t)std::min(knob, GRAM_SHARED_WAVES) * sms / items, m / 32);
+  want = std::max<int64_t>(1, want);
   if (max_splits > 0) want = std::min<int64_t>(want, max_splits);
   g.rows_per_split = ceil_div(ceil_div(m, want), row_unit) * row_unit;
   g.nsplit = std::max<int64_t>(1, ceil_div(m, g.rows_per_split));
   return g;
+}
+
+int64_t gram_split_capacity(int n, bool shared) {
+  const int per_sm = shared ? GRAM_SHARED_WAVES : gram_resident(n);
+  return std::max<int64_t>(1, (int64_t)per_sm * gram_sms() / gram_items((int)ceil_div(n, 128)));
 }
 
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g, double* partial,

@@ -29,9 +29,12 @@ struct GramGeom {
   size_t partial_doubles() const { return (size_t)nsplit * ntiles_total * T * T; }
 };
 // ctas_per_sm: most Gram CTAs per SM (an autotuned knob); row_unit: the ranges'
-// row counts are multiples of it; shared: for a shared lane (that
-// many waves of CTAs).
+// row counts are multiples of it; shared: for a shared lane (that many waves of
+// CTAs, up to GRAM_SHARED_WAVES).
+constexpr int GRAM_SHARED_WAVES = 4;
 GramGeom gram_geometry(int64_t m, int n, int64_t max_splits, int ctas_per_sm = 4, int row_unit = 4, bool shared = false);
+// The most ranges that gram_geometry returns for any m and knob.
+int64_t gram_split_capacity(int n, bool shared);
 cudaError_t gram_partials(const double* A, int64_t lda, int64_t m, int n, const GramGeom& g,
                           double* partial, Lane s);
 cudaError_t gram_reduce(const double* partial, const GramGeom& g, int n, double* W, int64_t ldw,
