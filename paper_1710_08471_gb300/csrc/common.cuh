@@ -77,12 +77,17 @@ __device__ __forceinline__ void grid_chain() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// Whether a grid of that many CTAs is set up early. One that fills the SMs is
-// not: while its predecessor holds some of them, its CTAs pile up on the rest.
+// Whether a grid of that many CTAs, each of some tens of microseconds or more
+// (Gram, Q-form, GEMM, Q^T b), is set up early. One that fills the SMs is not:
+// while its predecessor holds some of them, its CTAs pile up on the rest.
 // (777 columns in FP64: 15.4 ms, with every GEMM set up early 16.1. The Gram and
 // the Q-form pass twice their CTAs: these run for long on an SM each, and at
 // 4096 x 64 early ones cost 10 us. The 128 x 128 GEMMs of CholInv gain at up to
-// an SM each, 12 us of 2017 at 131601 x 256.)
+// an SM each, 12 us of 2017 at 131601 x 256.) Kernels whose CTAs last a
+// microsecond or so (sums of partials, packing, transposition, copies,
+// R2 R1) are set up early at any size: held to this rule too, 3000 x 80 took 235
+// us instead of 231, 4096 x 128 503 instead of 499, 8192 x 200 1668 instead of
+// 1657, and from 400 columns on nothing changed by more than 0.2%.
 inline bool chain_early(int64_t ctas) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
