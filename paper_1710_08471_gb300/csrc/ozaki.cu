@@ -1123,17 +1123,20 @@ bool oz_qform_wide(int n) {
 
 // Row ranges of the Gram: its items (ranges x tiles) all cost the same and are
 // dealt to the CTAs in whole rounds, so the ranges are chosen to fill the
-// rounds: the fewest rounds, up to four, that leave less than 5% of the CTAs
+// rounds: the fewest rounds, up to eight, that leave less than 5% of the CTAs
 // idle, or else the count that leaves the fewest. (Two items per CTA whatever
-// the tiles, as before, made three rounds of 2.1 at n = 200 and n = 512, a third
-// of the time idle: 2^21 x 512 15.5 -> 11.1 ms per Gram, 1000037 x 200 with six
-// slices 1.82 -> 1.36.)
+// the tiles made three rounds of 2.1 at n = 200 and n = 512, a third of the time
+// idle: 2^21 x 512 15.5 -> 11.1 ms per Gram, 1000037 x 200 with six slices 1.82 ->
+// 1.36. us for both Grams with up to 4, 8 and 16 rounds: 90000 x 1500 4811, 4181,
+// 4070; 200000 x 704 2002, 1966, 1966; 65536 x 2048 5274, 5276, 4847; 8192 x 1500
+// 545, 533, 574: the shorter ranges of many rounds cost few rows, and every
+// round another n x n partial per tile row of workspace, 110 MB more at 16.)
 int64_t oz_split_target(int n) {
   const int64_t units = sm_count_oz();
   const int tiles = oz_gram_tiles(n);
   int64_t best = 1;
   double best_use = 0.0;
-  for (int r = 1; r <= 4; ++r) {
+  for (int r = 1; r <= 8; ++r) {
     const int64_t splits = std::max<int64_t>(1, r * units / tiles), items = splits * tiles;
     const double use = (double)items / ((double)ceil_div(items, units) * units);
     if (use > best_use + 1e-9) {
