@@ -569,7 +569,8 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];  // 128-byte swizzle: 1024-byte atoms
   uint8_t* smem = smem_raw;
   // Kept as a value: with the base folded into every address as a constant the
-  // issuing thread's loop came out slower (Gram +1.5%).
+  // 64-column Q-form came out slower (2^27 entries, both: n = 512 2.98 -> 3.05 ms,
+  // 256 1.82 -> 1.85; the 32-column one 1.34 -> 1.32 at n = 64; the Gram the same).
   asm volatile("" : "+l"(smem));
   uint8_t* sA = smem;                  // NA slots
   uint8_t* sB = sA + NA * A_BYTES;     // 2 buffers x S planes
@@ -734,7 +735,8 @@ __global__ void __launch_bounds__(OzCfg<S, MODE, BN, EPI, NGRP>::THREADS, 1)
             // per 8 rows throughout) and group g = s + t is the BN-column
             // accumulator at column BN g, so each product lands in its group.
             // The S - s products of slice s go in as few MMAs as N <= 256
-            // allows, split evenly: short ones (N < 192) do not run at full rate.
+            // allows, split evenly (N = 256 first, then the rest: Gram of 2^27
+            // entries at n = 512 1.43 -> 1.49 ms, 64-column Q-form 1.53 -> 1.55).
             constexpr int NMMA_MAX = (S + C::TMAX - 1) / C::TMAX;
 #pragma unroll
             for (int q = 0, t0 = 0; q < NMMA_MAX && t0 < S - s; ++q) {
