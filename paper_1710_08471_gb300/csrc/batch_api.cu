@@ -16,6 +16,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <string>
 #include <vector>
 
@@ -37,7 +38,7 @@ struct cqr2_batch_st {
   BatchStatus* h_status = nullptr;
   DevStatus* d_lstatus = nullptr;  // status words of the planned problems
   DevStatus* h_lstatus = nullptr;
-  std::vector<cudaStream_t> side;
+  std::vector<cudaStream_t> side;  // cfg.streams for planned problems, then one for the grouped kernel's small size
   cudaEvent_t fork = nullptr;
   std::vector<cudaEvent_t> joins;
   struct PlanSlot {
@@ -119,18 +120,27 @@ cqr2_status_t batch_enqueue(cqr2_batch_t b, const cqr2_problem_t* problems, int3
   // The side streams fork here, ahead of the grouped launches, so that the
   // planned problems run beside them and not after them (a burst of 48 requests
   // with one in the grouped kernel waited 2.2 ms of its 37 for that one). The
-  // kernel's large size runs on the batch stream, its small size too, or on
-  // the first side stream if both are needed.
+  // kernel's large size runs on the batch stream, its small size too, or on a
+  // side stream of its own if both are needed: ahead of planned problems on one
+  // of theirs it held these up (200 x (8192 x 24), 100 x (8192 x 48) and 12 x
+  // (65536 x 128) in split precision 15.4 ms on four side streams, now 14.3; 20.2
+  // on one, now 17.4).
   const size_t narrow = small.size() - wide;
-  const bool both = wide > 0 && narrow > 0;
-  const int ns = (int)std::min<size_t>(b->side.size(), large.size()), nforked = std::max(ns, both ? 1 : 0);
-  if (nforked > 0 && cudaEventRecord(b->fork, b->stream) != cudaSuccess) return CQR2_ERR_CUDA;
-  for (int s = 0; s < nforked; ++s)
+  const int ns = (int)std::min<size_t>(b->cfg.streams, large.size());
+  std::vector<int> forked(ns);
+  std::iota(forked.begin(), forked.end(), 0);
+  cudaStream_t narrow_stream = b->stream;
+  if (wide > 0 && narrow > 0) {
+    narrow_stream = b->side.back();
+    forked.push_back((int)b->side.size() - 1);
+  }
+  if (!forked.empty() && cudaEventRecord(b->fork, b->stream) != cudaSuccess) return CQR2_ERR_CUDA;
+  for (int s : forked)
     if (cudaStreamWaitEvent(b->side[s], b->fork, 0) != cudaSuccess) return CQR2_ERR_CUDA;
   if (wide > 0 && cqr2_small_batched(b->d_probs, (int)wide, b->d_next, b->d_status, false, b->stream) != cudaSuccess)
     return CQR2_ERR_CUDA;
   if (narrow > 0 && cqr2_small_batched(b->d_probs + wide, (int)narrow, b->d_next + 1, b->d_status + wide, true,
-                                       both ? b->side[0] : b->stream) != cudaSuccess)
+                                       narrow_stream) != cudaSuccess)
     return CQR2_ERR_CUDA;
   b->last_small = small;
   // the others: plans on the side streams
@@ -165,7 +175,7 @@ cqr2_status_t batch_enqueue(cqr2_batch_t b, const cqr2_problem_t* problems, int3
       b->last_used.push_back(large[k]);
     }
   }
-  for (int s = 0; s < nforked; ++s) {
+  for (int s : forked) {
     if (cudaEventRecord(b->joins[s], b->side[s]) != cudaSuccess) return CQR2_ERR_CUDA;
     if (cudaStreamWaitEvent(b->stream, b->joins[s], 0) != cudaSuccess) return CQR2_ERR_CUDA;
   }
@@ -269,7 +279,7 @@ cqr2_status_t cqr2_batch_create(cqr2_batch_t* batch, int32_t max_count, int32_t 
             cudaMallocHost(&b->h_lstatus, sizeof(DevStatus) * max_count) == cudaSuccess &&
             cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) == cudaSuccess &&
             cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; ok && i < b->cfg.streams; ++i) {
+  for (int i = 0; ok && i <= b->cfg.streams; ++i) {
     cudaStream_t s;
     cudaEvent_t e;
     ok = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
