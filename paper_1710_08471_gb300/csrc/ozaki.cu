@@ -1128,7 +1128,7 @@ bool oz_qform_wide(int n) {
 // rounds: the fewest rounds, up to eight, that leave less than 5% of the CTAs
 // idle, or else the count that leaves the fewest. (Two items per CTA whatever
 // the tiles made three rounds of 2.1 at n = 200 and n = 512, a third of the time
-// idle: 2^21 x 512 15.5 -> 11.1 ms per Gram, 1000037 x 200 with six slices 1.82 ->
+// idle: 2^21 x 512 15.5 -> 11.4 ms per Gram, 1000037 x 200 with six slices 1.82 ->
 // 1.36. us for both Grams with up to 4, 8 and 16 rounds: 90000 x 1500 4811, 4181,
 // 4070; 200000 x 704 2002, 1966, 1966; 65536 x 2048 5274, 5276, 4847; 8192 x 1500
 // 545, 533, 574: the shorter ranges of many rounds cost few rows, and every
