@@ -1131,8 +1131,8 @@ bool oz_qform_wide(int n) {
 // idle: 2^21 x 512 15.5 -> 11.4 ms per Gram, 1000037 x 200 with six slices 1.82 ->
 // 1.36. us for both Grams with up to 4, 8 and 16 rounds: 90000 x 1500 4811, 4181,
 // 4070; 200000 x 704 2002, 1966, 1966; 65536 x 2048 5274, 5276, 4847; 8192 x 1500
-// 545, 533, 574: the shorter ranges of many rounds cost few rows, and every
-// round another n x n partial per tile row of workspace, 110 MB more at 16.)
+// 545, 533, 574: few rows lose more by the shorter ranges of 16 rounds than by
+// idle CTAs, and the partials of those take 110 MB more at n = 1500.)
 int64_t oz_split_target(int n) {
   const int64_t units = sm_count_oz();
   const int tiles = oz_gram_tiles(n);
