@@ -62,13 +62,13 @@ GB300_SMS = 152
 # "tall" entries were captured on "mid" (2^20 of the 2^23 rows) and scaled by
 # the row count: these kernels stream their operands once per launch.
 NCU_TRAFFIC = {
-    "k_qform_gram_small@mid@32201450a5426255": 2145473280,
-    "k_qform_gram_small@tall@32201450a5426255": 17163786240,
-    "k_ozaki_gemm<7,QFORM>@mid@f33dc9b14d75de37": 2938640128,
-    "k_ozaki_gemm<7,QFORM>@tall@f33dc9b14d75de37": 23509121024,
-    "k_ozaki_gemm<7,GRAM>@mid@f33dc9b14d75de37": 1892780800,
-    "k_ozaki_gemm<7,GRAM>@tall@f33dc9b14d75de37": 15142246400,
-    "k_cqr2_small_batched@batch@c56aa36f0d944e5a": 5306968320,
+    "k_qform_gram_small@mid@9d1531f63443b349": 2111866880,
+    "k_qform_gram_small@tall@9d1531f63443b349": 16894935040,
+    "k_ozaki_gemm<7,QFORM>@mid@11daf3b467c2e5ab": 2942458000,
+    "k_ozaki_gemm<7,QFORM>@tall@11daf3b467c2e5ab": 23539664000,
+    "k_ozaki_gemm<7,GRAM>@mid@11daf3b467c2e5ab": 1883154000,
+    "k_ozaki_gemm<7,GRAM>@tall@11daf3b467c2e5ab": 15065232000,
+    "k_cqr2_small_batched@batch@320da96a3fb78dd3": 5299440384,
 }
 
 
