@@ -1,4 +1,4 @@
-"""Split-precision Gram where its row ranges fill more than four rounds of the SMs
+"""Split-precision Gram where its row ranges fill the SMs more than four times
 (704, 1500 and 1600 columns), from few rows to more than the ranges need, one plan
 for several row counts. The bound is the error-free split's own."""
 import numpy as np
